@@ -9,7 +9,7 @@
 #include <cstring>
 #include <type_traits>
 
-#include "h37_common.cuh"
+#include "h37_moments.cuh"
 #include "pair_io.cuh"
 #include "reduce.cuh"
 
@@ -30,6 +30,66 @@ inline h37::Model model_of(const Sim* s) {
   return m;
 }
 
+// The same for the sweeps, in the precision R they compute in.
+template <typename R>
+h37::MomentModel<R> moment_model(const Sim* s) {
+  const h37::Model b = model_of(s);
+  h37::MomentModel<R> m;
+  for (int n = 0; n < 5; ++n) m.no[n] = (R)-s->rates.w[n];
+  m.s = (R)h37::kS;
+  const double tau = s->storage == LBM_F32 || s->storage == LBM_F64 ? h37::basis_temperature(s->theta_ref * h37::kS) : 0.0;
+  m.basis = (R)tau;
+  m.basis2x3 = (R)(3.0 * tau * tau);
+  m.th_ref = (R)(s->theta_ref * h37::kS - tau);
+  m.th_iso = (R)(h37::kS - tau);
+  m.kext = b.raw ? R(1) : R(1) - (R)b.kfac;
+  m.usq_max = (R)(4.0 * h37::kS);
+  m.thermal = b.thermal;
+  m.raw = b.raw;
+  m.sround = b.sround;
+  m.seed = b.seed;
+  return m;
+}
+
+// What a sweep takes and how it updates a node (or pair), by storage type.  Plain
+// FP32 transforms (FP32 storage with LBM_FAST_TRANSFORMS) stay on the Hermite
+// tables: their errors recur every step, and the row sums in FP32 drift twice as
+// fast (2.0e-5 against 1.1e-5 relative on the velocity after 1000 steps).
+struct TableModel {
+  Rates r;
+  h37::Model m;
+};
+template <int S, bool EXACT>
+using SweepModel = typename std::conditional<S == LBM_F32 && !EXACT, TableModel,
+                                             h37::MomentModel<typename h37::Store<S>::calc>>::type;
+template <int S, bool EXACT>
+SweepModel<S, EXACT> sweep_model(const Sim* s) {
+  if constexpr (S == LBM_F32 && !EXACT)
+    return TableModel{s->rates, model_of(s)};
+  else
+    return moment_model<typename h37::Store<S>::calc>(s);
+}
+// mom, if not null: drho and the momentum in lattice units
+template <typename T, bool SCALED>
+__device__ __forceinline__ bool update_values(T (&v)[h37::kQ], const TableModel& t, T* mom) {
+  T om[5];
+#pragma unroll
+  for (int n = 0; n < 5; ++n) om[n] = cst<T>(t.r.w[n]);
+  const bool ok = h37::collide<T>(v, om, t.m, mom);
+  if (mom) {
+    mom[1] = mom[1] * cst<T>(1.0 / h37::kC);
+    mom[2] = mom[2] * cst<T>(1.0 / h37::kC);
+  }
+  return ok;
+}
+template <typename T, bool SCALED, typename R>
+__device__ __forceinline__ bool update_values(T (&v)[h37::kQ], const h37::MomentModel<R>& m, T* mom) {
+  return h37::collide_rows<T, SCALED, !SCALED>(v, m, mom);
+}
+template <typename R>
+__device__ __forceinline__ const h37::MomentModel<R>& rounding(const h37::MomentModel<R>& m) { return m; }
+__device__ __forceinline__ const h37::Model& rounding(const TableModel& t) { return t.m; }
+
 inline h37::Grid2 grid2(const Sim* s) { return h37::Grid2{(int)s->nx, (int)s->ny, s->N}; }
 
 // LBM_H37_SWEEP=scalar keeps the one-node kernel for every storage type (read at
@@ -45,33 +105,65 @@ inline bool h37_scalar_only() {
   return e && std::strcmp(e, "scalar") == 0;
 }
 
+// Stored value to the number the node update takes, and back (the update works on
+// f / w where that is what is stored).
+template <int S>
+__device__ __forceinline__ typename h37::Store<S>::calc unstore(typename h37::Store<S>::type s) {
+  if constexpr (S == LBM_F16)
+    return __half2float(s);
+  else if constexpr (S == LBM_BF16)
+    return __bfloat162float(s);
+  else
+    return s;
+}
+template <int S>
+__device__ __forceinline__ typename h37::Store<S>::type restore(typename h37::Store<S>::calc v) {
+  if constexpr (S == LBM_F16)
+    return __float2half_rn(v);
+  else if constexpr (S == LBM_BF16)
+    return __float2bfloat16_rn(v);
+  else
+    return v;
+}
+template <int S>
+__device__ __forceinline__ typename h37::Store<S>::type restore_sr(typename h37::Store<S>::calc v, uint32_t r) {
+  if constexpr (S == LBM_F16)
+    return __float2half_rz(h37::dither(v, r, 13));
+  else if constexpr (S == LBM_BF16)
+    return __float2bfloat16_rz(h37::dither(v, r, 16));
+  else
+    return v;
+}
+
 // EXACT: correctly rounded transforms (FP32 storage unless LBM_FAST_TRANSFORMS).
+// Threads walk the nodes of the grid in one dimension, so that rows of any
+// length fill the warps.
 template <int S, bool ODD, bool EXACT>
 __global__ void __launch_bounds__(kH37Threads)
-    h37_sweep_kernel(typename h37::Store<S>::type* __restrict__ f, h37::Grid2 g, Rates r, h37::Model m,
-                     int* __restrict__ status) {
+    h37_sweep_kernel(typename h37::Store<S>::type* __restrict__ f, h37::Grid2 g,
+                     SweepModel<S, EXACT> m, int* __restrict__ status) {
   using T = typename h37::Store<S>::calc;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= g.nx) return;
-  const int y = blockIdx.y;
-  T om[5];
-#pragma unroll
-  for (int n = 0; n < 5; ++n) om[n] = (T)r.w[n];
+  constexpr bool kScaled = S == LBM_F16 || S == LBM_BF16;
+  const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
+  if (node >= (uint32_t)g.N) return;
+  const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
   T v[h37::kQ];
-  h37::gather<S>(f, g, x, y, ODD ? 1 : 0, v);
-  const bool ok = h37::collide<T, EXACT>(v, om, m);
+#pragma unroll
+  for (int j = 0; j < h37::kQ; ++j)
+    v[ODD ? h37::opp(j) : j] = unstore<S>(f[(size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : node)]);
+  bool ok;
+  if constexpr (EXACT)
+    ok = h37::collide_exact(v, m);
+  else
+    ok = update_values<T, kScaled>(v, m, static_cast<T*>(nullptr));
   if (!ok) atomicOr(status, 1);
   // even sweep: population i goes to slot (x, opp(i)); odd sweep: to slot (x + e_i, i)
-  const uint32_t node = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
-  h37::SrStream rs(m.seed, node);
+  h37::SrStream rs(rounding(m).seed, node);
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j) {
     const T val = ODD ? v[j] : v[h37::opp(j)];
-    const auto e = m.sround ? h37::encode_sr<S>(val, j, rs.next()) : h37::encode<S>(val, j);
-    if (!ODD)
-      f[(size_t)j * g.N + node] = e;
-    else
-      f[(size_t)j * g.N + h37::nbr(g, x, y, j)] = e;
+    const auto e = kScaled && rounding(m).sround ? restore_sr<S>(val, rs.next()) : restore<S>(val);
+    f[(size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : node)] = e;
   }
 }
 
@@ -86,11 +178,11 @@ __global__ void __launch_bounds__(kH37Threads)
 #define LBM_H37_PAIR_MINB 3  // 168 registers (a few words spill): 12 warps per SM
 #endif
 // The update of pair xp of row blockIdx.y; with TOT the pair's conserved
-// moments (drho, j_x, j_y in Hermite units, both lanes) go to mom[0..2].
+// moments (drho, j_x, j_y, both lanes) go to mom[0..2].
 template <int S, bool ODD, bool TOT>
 __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restrict__ f, const h37::Grid2& g,
-                                                const Rates& r, const h37::Model& m, int* __restrict__ status,
-                                                int xp, f2* mom) {
+                                                const SweepModel<S, false>& m, int* __restrict__ status, int xp,
+                                                f2* mom) {
   using IO = PairIO<S>;
   using E = typename IO::E;
   const int y = blockIdx.y;
@@ -102,9 +194,6 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
     yy = yy < 0 ? yy + g.ny : (yy >= g.ny ? yy - g.ny : yy);
     return (uint32_t)nx * (uint32_t)yy;
   };
-  f2 om[5];
-#pragma unroll
-  for (int n = 0; n < 5; ++n) om[n] = cst<f2>(r.w[n]);
   f2 v[h37::kQ];
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j) {
@@ -120,19 +209,17 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
       else
         val = IO::load11(fj + ro + wrapx(x0 + ex), fj + ro + wrapx(x0 + 1 + ex));
     }
-    if (IO::kScaled) val = val * cst<f2>(h37::w_of(j));
     v[ODD ? h37::opp(j) : j] = val;
   }
-  const bool ok = h37::collide<f2>(v, om, m, TOT ? mom : nullptr);
+  const bool ok = update_values<f2, IO::kScaled>(v, m, TOT ? mom : nullptr);
   if (!ok) atomicOr(status, 1);
   // the pair's own nodes (for the stochastic-rounding bits)
   const uint32_t n0 = (uint32_t)x0 + (uint32_t)nx * (uint32_t)y, n1 = (uint32_t)wrapx(x0 + 1) + (uint32_t)nx * (uint32_t)y;
-  h37::SrStream rs0(m.seed, n0), rs1(m.seed, n1);
+  h37::SrStream rs0(rounding(m).seed, n0), rs1(rounding(m).seed, n1);
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j) {
     E* fj = f + (size_t)j * g.N;
     f2 val = ODD ? v[j] : v[h37::opp(j)];
-    if (IO::kScaled) val = val * cst<f2>(1.0 / h37::w_of(j));
     E* pa;
     E* pb;
     bool adjacent;
@@ -148,7 +235,7 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
       adjacent = (ex & 1) != 0;
     }
     if constexpr (S == LBM_F16 || S == LBM_BF16) {
-      if (m.sround) {
+      if (rounding(m).sround) {
         float lo, hi;
         unpack2(val, lo, hi);
         const uint32_t r0 = rs0.next(), r1 = rs1.next();
@@ -171,11 +258,11 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
 
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
-    h37_pair_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, Rates r, h37::Model m,
+    h37_pair_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, SweepModel<S, false> m,
                     int* __restrict__ status) {
   const int xp = blockIdx.x * blockDim.x + threadIdx.x;
   if (2 * xp >= g.nx) return;
-  h37_pair_update<S, ODD, false>(f, g, r, m, status, xp, nullptr);
+  h37_pair_update<S, ODD, false>(f, g, m, status, xp, nullptr);
 }
 
 // The same sweep, which also writes the totals of the state it consumed (the
@@ -184,22 +271,17 @@ __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
 // partials[warp * 8 + k]; a warp sums its 64 nodes in FP32 (fixed shuffle tree).
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
-    h37_pair_totals_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, Rates r, h37::Model m,
+    h37_pair_totals_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, SweepModel<S, false> m,
                            int* __restrict__ status, float* __restrict__ partials) {
   const int xp = blockIdx.x * blockDim.x + threadIdx.x;
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   if (2 * xp < g.nx) {
     f2 mom[3];
-    h37_pair_update<S, ODD, true>(f, g, r, m, status, xp, mom);
-    const float ic = (float)(1.0 / h37::kC);
+    h37_pair_update<S, ODD, true>(f, g, m, status, xp, mom);
     float d0, d1, jx0, jx1, jy0, jy1;
     unpack2(mom[0], d0, d1);
     unpack2(mom[1], jx0, jx1);
     unpack2(mom[2], jy0, jy1);
-    jx0 *= ic;
-    jx1 *= ic;
-    jy0 *= ic;
-    jy1 *= ic;
     acc[0] = d0 + d1;
     acc[1] = jx0 + jx1;
     acc[2] = jy0 + jy1;
@@ -386,11 +468,9 @@ cudaError_t pair_t(Sim* s, int odd) {
   dim3 grid((unsigned)((s->nx / 2 + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
   E* f = static_cast<E*>(s->pop);
   if (odd)
-    h37_pair_kernel<S, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                    status_word(s));
+    h37_pair_kernel<S, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s));
   else
-    h37_pair_kernel<S, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                     status_word(s));
+    h37_pair_kernel<S, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s));
   return cudaGetLastError();
 }
 
@@ -400,12 +480,18 @@ cudaError_t pair_totals_t(Sim* s, int odd, float* partials) {
   dim3 grid((unsigned)((s->nx / 2 + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
   E* f = static_cast<E*>(s->pop);
   if (odd)
-    h37_pair_totals_kernel<S, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                           status_word(s), partials);
+    h37_pair_totals_kernel<S, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s), partials);
   else
-    h37_pair_totals_kernel<S, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                            status_word(s), partials);
+    h37_pair_totals_kernel<S, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s), partials);
   return cudaGetLastError();
+}
+
+// Threads per block of the one-node sweep: the largest of 128, 64, 32 that gives
+// every SM two blocks, so that small grids spread over all of them.
+inline int node_threads(int64_t N) {
+  int t = kH37Threads;
+  while (t > 32 && N < (int64_t)t * 2 * 152) t /= 2;
+  return t;
 }
 
 template <int S>
@@ -414,26 +500,19 @@ cudaError_t sweep_t(Sim* s, int odd) {
   if constexpr (S != LBM_F64) {
     if (h37_pair_supported(s)) return pair_t<S>(s, odd);
   }
-  dim3 grid((unsigned)((s->nx + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
+  const int t = node_threads(s->N);
+  const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   E* f = static_cast<E*>(s->pop);
+  auto launch = [&](auto odd_c, auto exact_c) {
+    h37_sweep_kernel<S, decltype(odd_c)::value, decltype(exact_c)::value>
+        <<<blocks, t, 0, s->stream>>>(f, grid2(s), sweep_model<S, decltype(exact_c)::value>(s), status_word(s));
+    return cudaGetLastError();
+  };
   if constexpr (S == LBM_F32) {
-    if (h37_exact_transforms(s)) {
-      if (odd)
-        h37_sweep_kernel<S, true, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                           status_word(s));
-      else
-        h37_sweep_kernel<S, false, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                            status_word(s));
-      return cudaGetLastError();
-    }
+    if (h37_exact_transforms(s))
+      return odd ? launch(std::true_type(), std::true_type()) : launch(std::false_type(), std::true_type());
   }
-  if (odd)
-    h37_sweep_kernel<S, true, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                          status_word(s));
-  else
-    h37_sweep_kernel<S, false, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), s->rates, model_of(s),
-                                                                           status_word(s));
-  return cudaGetLastError();
+  return odd ? launch(std::true_type(), std::false_type()) : launch(std::false_type(), std::false_type());
 }
 
 template <int S>

@@ -182,58 +182,6 @@ __device__ __forceinline__ float two_sum_err(float a, float b, float s) {
   return (a - (s - z)) + (b - z);
 }
 
-__device__ __forceinline__ void to_hermite_exact(const float (&v)[kQ], float (&a)[kNC]) {
-  float sp[kHalf], dm[kHalf], spe[kHalf], dme[kHalf];
-#pragma unroll
-  for (int i = 0; i < kHalf; ++i) {
-    sp[i] = v[i] + v[opp(i)];
-    dm[i] = v[i] - v[opp(i)];
-    spe[i] = two_sum_err(v[i], v[opp(i)], sp[i]);
-    dme[i] = two_sum_err(v[i], -v[opp(i)], dm[i]);
-  }
-#pragma unroll
-  for (int c = 0; c < kNC; ++c) {
-    const bool even = (corder(c) & 1) == 0;
-    float s = 0.f, cc = 0.f;
-    if (even) dot2_add(s, cc, v[kHalf], hval(kHalf, c));
-#pragma unroll
-    for (int i = 0; i < kHalf; ++i) {
-      const double h = hval(i, c);
-      if (h == 0.0) continue;
-      dot2_add(s, cc, even ? sp[i] : dm[i], h);
-      cc = __fmaf_rn(even ? spe[i] : dme[i], (float)h, cc);  // the pair sum's own rounding
-    }
-    a[c] = s + cc;
-  }
-}
-
-__device__ __forceinline__ void from_hermite_exact(const float (&a)[kNC], float (&v)[kQ]) {
-  {
-    float s = 0.f, cc = 0.f;
-#pragma unroll
-    for (int c = 0; c < kNC; ++c)
-      if ((corder(c) & 1) == 0 && rval(kHalf, c) != 0.0) dot2_add(s, cc, a[c], rval(kHalf, c));
-    v[kHalf] = s + cc;
-  }
-#pragma unroll
-  for (int i = 0; i < kHalf; ++i) {
-    float ev = 0.f, evc = 0.f, od = 0.f, odc = 0.f;
-#pragma unroll
-    for (int c = 0; c < kNC; ++c) {
-      const double r = rval(i, c);
-      if (r == 0.0) continue;
-      if ((corder(c) & 1) == 0)
-        dot2_add(ev, evc, a[c], r);
-      else
-        dot2_add(od, odc, a[c], r);
-    }
-    // v_i, v_opp(i) = (ev + evc) +- (od + odc), the corrections folded in before the last rounding
-    const float t1 = ev + od, t2 = ev - od;
-    v[i] = t1 + (two_sum_err(ev, od, t1) + (evc + odc));
-    v[opp(i)] = t2 + (two_sum_err(ev, -od, t2) + (evc - odc));
-  }
-}
-
 // rho > 0, theta = 1 + eps > 0 and |u|^2 < 4 (Hermite units), for every node held.
 __device__ __forceinline__ bool physical(float rho, float eps, float usq) {
   return rho > 0.f && 1.f + eps > 0.f && usq < 4.f;
@@ -389,25 +337,17 @@ __device__ __forceinline__ bool collide_coeffs(T (&da)[NC], const T (&om)[5], co
 
 // One node of the 37-velocity lattice.  v: offsets f_i - f_ref,i in,
 // post-collision offsets out.  om[n]: rates of orders 2..4.
-// EXACT (FP32 only): the correctly rounded transforms above.
-template <typename T, bool EXACT = false>
+template <typename T>
 __device__ __forceinline__ bool collide(T (&v)[kQ], const T (&om)[5], const Model& m, T* mom = nullptr) {
-  static_assert(!EXACT || std::is_same<T, float>::value, "correctly rounded transforms are FP32");
   T da[kNC];
-  if constexpr (EXACT)
-    to_hermite_exact(v, da);
-  else
-    to_hermite<T>(v, da);
+  to_hermite<T>(v, da);
   if (mom) {  // the node's conserved moments: drho and j (Hermite units), unchanged by the collision
     mom[0] = da[0];
     mom[1] = da[cidx(1, 0)];
     mom[2] = da[cidx(0, 1)];
   }
   const bool ok = collide_coeffs<T, kNC>(da, om, m);
-  if constexpr (EXACT)
-    from_hermite_exact(da, v);
-  else
-    from_hermite<T>(da, v);
+  from_hermite<T>(da, v);
   return ok;
 }
 

@@ -414,3 +414,43 @@ def test_full_size_thermal_1024_fp16_one_step_bound(lbm):
         bound = w_lib * 2.0 ** -11 * np.abs((fo - fref) / w_lib) * 1.05 + 2e-7
         assert np.all(np.abs(g - fo) <= bound), np.max(np.abs(g - fo) / bound)
     assert sim.status() == 0
+
+
+# copies of a 7 x 5 pattern: N on both sides of the block-size switches (32, 64 and
+# 128 threads at fewer or more than 9728, 19456 and 38912 nodes), none a multiple of a warp
+@pytest.mark.parametrize("copies", [(1, 2), (19, 14), (19, 15), (37, 15), (37, 16), (75, 15), (79, 15)])
+@pytest.mark.parametrize("storage,thermal", [("f64", True), ("f32", True), ("f32", False), ("f16", True)])
+def test_a_tiled_pattern_evolves_as_one_copy_bit_for_bit(lbm, storage, thermal, copies):
+    """A node's update does not depend on where it is: a grid of identical periodic
+    copies holds the same bits in every copy as the single copy's own run, for
+    every grid size (blocks, remainders) and both parities."""
+    base = (7, 5)
+    rho, u, theta = _fields(base, seed=3)
+    if not thermal:
+        theta = np.ones_like(theta)
+    tile = lambda q: np.tile(q.reshape(base[1], base[0]), (copies[1], copies[0])).reshape(-1)
+    a = _sim(lbm, base, TAUS, storage, thermal)
+    b = _sim(lbm, (base[0] * copies[0], base[1] * copies[1]), TAUS, storage, thermal)
+    a.init_fields(rho, u, theta)
+    b.init_fields(tile(rho), np.stack([tile(u[0]), tile(u[1])]), tile(theta))
+    for _ in range(3):
+        a.step(1)
+        b.step(1)
+        pa, pb = a.populations(), b.populations()
+        want = np.stack([tile(q) for q in pa])
+        assert np.array_equal(pb, want)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, -3.0])
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16"])
+def test_an_unphysical_node_is_flagged(lbm, storage, bad):
+    """NaN, infinities and a negative density reach the status word of every sweep."""
+    dims = (10, 6)
+    rho, u, theta = _fields(dims, seed=3)
+    sim = _sim(lbm, dims, TAUS, storage)
+    sim.init_fields(rho, u, theta)
+    f = sim.populations()
+    f[18, 23] = bad
+    sim.set_populations(f)
+    sim.step(1)
+    assert sim.status() == lbm.LBM_EDIVERGED
