@@ -630,15 +630,27 @@ __device__ __forceinline__ void to_polynomial_exact(const float (&M)[NC], const 
   put(i11, b11);
 }
 
+// hi + lo parts of the sums as M + L, M rounded
+template <int NC>
+__device__ __forceinline__ void round_parts(const f2 (&M2)[NC], float (&M)[NC], float (&L)[NC]) {
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    float hi, lo;
+    unpack2(M2[k], hi, lo);
+    M[k] = hi + lo;
+    L[k] = lo - (M[k] - hi);
+  }
+}
+
 constexpr int kMomentBits = 10;      // sum of e_x^4 over the rule: 660
 constexpr int kPolynomialBits = 8;   // sum of |e_x^p e_y^q| over p + q <= 4 at (3, 1): 179
 
 template <int NC>
-__device__ __forceinline__ void cut_polynomial(const float (&s)[NC], const float (&c)[NC], f2 (&b)[NC]) {
+__device__ __forceinline__ void cut_polynomial(const float (&s)[NC], const float (&c)[NC], f2 (&b)[NC], int bits) {
   float mx = fabsf(s[0]);
 #pragma unroll
   for (int k = 1; k < NC; ++k) mx = fmaxf(mx, fabsf(s[k]));
-  const float sigma = cut_at(mx, kPolynomialBits);
+  const float sigma = cut_at(mx, bits);
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
     float hi, lo;
@@ -719,13 +731,7 @@ __device__ __forceinline__ bool collide_exact(float (&v)[kQ], const MomentModel<
 #pragma unroll
     for (int i = 0; i < kQ; ++i) x[i] = cut(v[i], sigma);
     to_moments<f2, false>(x, M2);
-#pragma unroll
-    for (int k = 0; k < kNC; ++k) {
-      float hi, lo;
-      unpack2(M2[k], hi, lo);
-      M[k] = hi + lo;
-      L[k] = lo - (M[k] - hi);
-    }
+    round_parts<kNC>(M2, M, L);
   }
   float H[kNC];
   to_basis_exact<kNC>(M, L, H, m);
@@ -733,7 +739,7 @@ __device__ __forceinline__ bool collide_exact(float (&v)[kQ], const MomentModel<
   add_increments<kNC>(M, L, inc);
   to_polynomial_exact<kNC>(M, L, BuiltInSplitMap(), s, c);
   f2 b[kNC], x[kQ];
-  cut_polynomial<kNC>(s, c, b);
+  cut_polynomial<kNC>(s, c, b, kPolynomialBits);
   from_polynomial<f2, true>(b, x);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) v[i] = weigh(x[i], split_of(w_of(i)));

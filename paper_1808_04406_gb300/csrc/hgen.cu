@@ -5,13 +5,17 @@
 // same Hermite-space CM-MRT as on the built-in 37-velocity lattice
 // (h37::collide_coeffs: Eq. omega in the relative frame, K = 6 at order 4);
 // only the projection onto and from the Hermite coefficients differs: it uses
-// per-simulation tables (HTables) passed by value instead of compiled-in
-// constants.  One node per thread, AA pattern, FP64 or FP32 offsets from
-// f_eq(1, 0, theta_ref).  Velocities crossing the C ABI are in lattice units.
+// per-simulation tables passed by value instead of compiled-in constants.  One
+// node per thread, AA pattern, FP64 or FP32 offsets from f_eq(1, 0, theta_ref).
+// Velocities crossing the C ABI are in lattice units.
+//
+// Rules that are symmetric under e_x -> -e_x and e_y -> -e_y (every minimal rule
+// is) go through hgen_orbit_kernel: raw moments of the reflection orbits.  Others,
+// and plain FP32 transforms, take the dense tables (hgen_sweep_kernel).
 #include <cmath>
 #include <type_traits>
 
-#include "h37_common.cuh"
+#include "h37_moments.cuh"
 #include "reduce.cuh"
 
 namespace lbm {
@@ -205,6 +209,358 @@ __global__ void __launch_bounds__(kHgThreads)
   }
 }
 
+// ---- reflection orbits --------------------------------------------------------
+// The velocities of a rule with both reflections are the rest velocity, pairs
+// (+-a, 0) and (0, +-a), and quadruples (+-a, +-b).  The raw moments M_pq (lattice
+// units; h37_moments.cuh has the collision on them) need each orbit only as its
+// sums of even and odd parity in x and y: with 37 velocities and N = 4 that takes
+// 180 FP64 operations in and 181 out, against 555 each way through the dense
+// tables, which bound this kernel (FP64 runs at 1 / 76 of the FP32 rate).
+// Shear wave on 80^2, rule E9-A, FP64: 48.2 -> 24.6 us a step (of which 18 are the FP64 pipe: one warp on each of
+// 200 of the 608 SM partitions, 64 cycles per FP64 warp instruction).
+template <typename T, int NA, int NQ>
+struct Orbits {
+  int rest, xp[NA], xm[NA], yp[NA], ym[NA], pp[NQ], mp[NQ], pm[NQ], mm[NQ];  // velocity indices
+  int da[NA], qa[NQ], qb[NQ];                                                // |e| of pairs, |e_x| and |e_y| of quadruples
+  T w0, pw[NA], qw[NQ];                                                      // weights (1 where a sum is weighted later)
+  T p1[NA], p2[NA], p3[NA], p4[NA];                                          // powers of a
+  T a1[NQ], a2[NQ], a3[NQ], a4[NQ], b1[NQ], b2[NQ], b3[NQ], b4[NQ];          // a^p b^q of quadruples
+  T ab[NQ], a2b[NQ], ab2[NQ], a2b2[NQ], a3b[NQ], ab3[NQ];
+  T vp1[NA], vp2[NA], vp3[NA], vp4[NA];  // the same times the weight
+  T va1[NQ], va2[NQ], va3[NQ], va4[NQ], vb1[NQ], vb2[NQ], vb3[NQ], vb4[NQ];
+  T vab[NQ], va2b[NQ], vab2[NQ], va2b2[NQ], va3b[NQ], vab3[NQ];
+};
+
+// Fills o from the rule; false if the rule lacks a reflection, has other numbers of
+// orbits, or weights that differ within an orbit.  weighted = false: weights of 1.
+template <typename T, int NA, int NQ>
+bool make_orbits(const HLattice& L, bool weighted, Orbits<T, NA, NQ>* o) {
+  int at[7][7];
+  for (auto& r : at)
+    for (int& k : r) k = -1;
+  for (int i = 0; i < L.q; ++i) at[L.ey[i] + 3][L.ex[i] + 3] = i;
+  auto idx = [&](int x, int y) { return at[y + 3][x + 3]; };
+  auto same = [&](int i, int j) { return i >= 0 && j >= 0 && L.w[i] == L.w[j]; };
+  int na = 0, nq = 0;
+  o->rest = idx(0, 0);
+  if (o->rest < 0) return false;
+  o->w0 = weighted ? (T)L.w[o->rest] : T(1);
+  for (int a = 1; a <= 3; ++a) {
+    const int xp = idx(a, 0), xm = idx(-a, 0), yp = idx(0, a), ym = idx(0, -a);
+    if (xp < 0 && xm < 0 && yp < 0 && ym < 0) continue;
+    if (!same(xp, xm) || !same(yp, ym) || !same(xp, yp) || na == NA) return false;
+    o->xp[na] = xp;
+    o->xm[na] = xm;
+    o->yp[na] = yp;
+    o->ym[na] = ym;
+    o->da[na] = a;
+    const double w = weighted ? L.w[xp] : 1.0, d = a;
+    o->pw[na] = (T)w;
+    o->p1[na] = (T)d;
+    o->p2[na] = (T)(d * d);
+    o->p3[na] = (T)(d * d * d);
+    o->p4[na] = (T)(d * d * d * d);
+    o->vp1[na] = (T)(w * d);
+    o->vp2[na] = (T)(w * d * d);
+    o->vp3[na] = (T)(w * d * d * d);
+    o->vp4[na] = (T)(w * d * d * d * d);
+    ++na;
+  }
+  for (int b = 1; b <= 3; ++b)
+    for (int a = 1; a <= 3; ++a) {
+      const int pp = idx(a, b), mp = idx(-a, b), pm = idx(a, -b), mm = idx(-a, -b);
+      if (pp < 0 && mp < 0 && pm < 0 && mm < 0) continue;
+      if (!same(pp, mp) || !same(pp, pm) || !same(pp, mm) || nq == NQ) return false;
+      const int k = nq++;
+      o->pp[k] = pp;
+      o->mp[k] = mp;
+      o->pm[k] = pm;
+      o->mm[k] = mm;
+      o->qa[k] = a;
+      o->qb[k] = b;
+      const double w = weighted ? L.w[pp] : 1.0, x = a, y = b;
+      o->qw[k] = (T)w;
+      o->a1[k] = (T)x;
+      o->a2[k] = (T)(x * x);
+      o->a3[k] = (T)(x * x * x);
+      o->a4[k] = (T)(x * x * x * x);
+      o->b1[k] = (T)y;
+      o->b2[k] = (T)(y * y);
+      o->b3[k] = (T)(y * y * y);
+      o->b4[k] = (T)(y * y * y * y);
+      o->ab[k] = (T)(x * y);
+      o->a2b[k] = (T)(x * x * y);
+      o->ab2[k] = (T)(x * y * y);
+      o->a2b2[k] = (T)(x * x * y * y);
+      o->a3b[k] = (T)(x * x * x * y);
+      o->ab3[k] = (T)(x * y * y * y);
+      o->va1[k] = (T)(w * x);
+      o->va2[k] = (T)(w * x * x);
+      o->va3[k] = (T)(w * x * x * x);
+      o->va4[k] = (T)(w * x * x * x * x);
+      o->vb1[k] = (T)(w * y);
+      o->vb2[k] = (T)(w * y * y);
+      o->vb3[k] = (T)(w * y * y * y);
+      o->vb4[k] = (T)(w * y * y * y * y);
+      o->vab[k] = (T)(w * x * y);
+      o->va2b[k] = (T)(w * x * x * y);
+      o->vab2[k] = (T)(w * x * y * y);
+      o->va2b2[k] = (T)(w * x * x * y * y);
+      o->va3b[k] = (T)(w * x * x * x * y);
+      o->vab3[k] = (T)(w * x * y * y * y);
+    }
+  return na == NA && nq == NQ && 1 + 4 * NA + 4 * NQ == L.q;
+}
+
+// Node values by orbit, and calls of fn(value, velocity index, signed e_x, signed e_y, index of
+// the opposite velocity) for each.
+template <typename T, int NA, int NQ>
+struct OrbitValues {
+  T r, xp[NA], xm[NA], yp[NA], ym[NA], pp[NQ], mp[NQ], pm[NQ], mm[NQ];
+  template <typename R, typename F>
+  __device__ __forceinline__ void each(const Orbits<R, NA, NQ>& o, F fn) {
+    fn(r, o.rest, 0, 0, o.rest);
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+      fn(xp[k], o.xp[k], o.da[k], 0, o.xm[k]);
+      fn(xm[k], o.xm[k], -o.da[k], 0, o.xp[k]);
+      fn(yp[k], o.yp[k], 0, o.da[k], o.ym[k]);
+      fn(ym[k], o.ym[k], 0, -o.da[k], o.yp[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) {
+      fn(pp[k], o.pp[k], o.qa[k], o.qb[k], o.mm[k]);
+      fn(mp[k], o.mp[k], -o.qa[k], o.qb[k], o.pm[k]);
+      fn(pm[k], o.pm[k], o.qa[k], -o.qb[k], o.mp[k]);
+      fn(mm[k], o.mm[k], -o.qa[k], -o.qb[k], o.pp[k]);
+    }
+  }
+};
+
+// T: the values' type (f2: hi and lo parts), R: that of the constants
+template <typename T, typename R, int NA, int NQ, int NC>
+__device__ __forceinline__ void orbit_moments(const Orbits<R, NA, NQ>& o, const OrbitValues<T, NA, NQ>& v,
+                                              T (&M)[NC]) {
+  using h37::cidx;
+  using h37::spread;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) M[c] = cst<T>(0.0);
+  M[0] = v.r;
+  auto acc = [&](int c, R k, T x) { M[c] = fma_(spread<T>(k), x, M[c]); };
+#pragma unroll
+  for (int k = 0; k < NQ; ++k) {
+    const T s1 = v.pp[k] + v.mm[k], d1 = v.pp[k] - v.mm[k], s2 = v.pm[k] + v.mp[k], d2 = v.pm[k] - v.mp[k];
+    const T ee = s1 + s2, oo = s1 - s2, oe = d1 + d2, eo = d1 - d2;
+    M[0] = M[0] + ee;
+    acc(cidx(2, 0), o.a2[k], ee);
+    acc(cidx(0, 2), o.b2[k], ee);
+    acc(cidx(1, 0), o.a1[k], oe);
+    acc(cidx(3, 0), o.a3[k], oe);
+    acc(cidx(1, 2), o.ab2[k], oe);
+    acc(cidx(0, 1), o.b1[k], eo);
+    acc(cidx(0, 3), o.b3[k], eo);
+    acc(cidx(2, 1), o.a2b[k], eo);
+    acc(cidx(1, 1), o.ab[k], oo);
+    if constexpr (NC == 15) {
+      acc(cidx(4, 0), o.a4[k], ee);
+      acc(cidx(0, 4), o.b4[k], ee);
+      acc(cidx(2, 2), o.a2b2[k], ee);
+      acc(cidx(3, 1), o.a3b[k], oo);
+      acc(cidx(1, 3), o.ab3[k], oo);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    const T sx = v.xp[k] + v.xm[k], dx = v.xp[k] - v.xm[k], sy = v.yp[k] + v.ym[k], dy = v.yp[k] - v.ym[k];
+    M[0] = M[0] + (sx + sy);
+    acc(cidx(1, 0), o.p1[k], dx);
+    acc(cidx(2, 0), o.p2[k], sx);
+    acc(cidx(3, 0), o.p3[k], dx);
+    acc(cidx(0, 1), o.p1[k], dy);
+    acc(cidx(0, 2), o.p2[k], sy);
+    acc(cidx(0, 3), o.p3[k], dy);
+    if constexpr (NC == 15) {
+      acc(cidx(4, 0), o.p4[k], sx);
+      acc(cidx(0, 4), o.p4[k], sy);
+    }
+  }
+}
+
+// w P(e) at every velocity (P(e) where the weights of o are 1)
+template <typename T, typename R, int NA, int NQ, int NC>
+__device__ __forceinline__ void orbit_values(const Orbits<R, NA, NQ>& o, const T (&b)[NC], OrbitValues<T, NA, NQ>& v,
+                                             bool weighted) {
+  using h37::cidx;
+  using h37::spread;
+  auto w0 = [&](R w, T x) { return weighted ? spread<T>(w) * x : x; };
+  auto add = [&](R k, int c, T x) { return fma_(spread<T>(k), b[c], x); };
+  auto mul = [&](R k, int c) { return spread<T>(k) * b[c]; };
+  v.r = w0(o.w0, b[0]);
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    const T z = w0(o.pw[k], b[0]);
+    T ex = add(o.vp2[k], cidx(2, 0), z), ey = add(o.vp2[k], cidx(0, 2), z);
+    if constexpr (NC == 15) {
+      ex = add(o.vp4[k], cidx(4, 0), ex);
+      ey = add(o.vp4[k], cidx(0, 4), ey);
+    }
+    const T ox = add(o.vp3[k], cidx(3, 0), mul(o.vp1[k], cidx(1, 0)));
+    const T oy = add(o.vp3[k], cidx(0, 3), mul(o.vp1[k], cidx(0, 1)));
+    v.xp[k] = ex + ox;
+    v.xm[k] = ex - ox;
+    v.yp[k] = ey + oy;
+    v.ym[k] = ey - oy;
+  }
+#pragma unroll
+  for (int k = 0; k < NQ; ++k) {
+    T ee = add(o.va2[k], cidx(2, 0), add(o.vb2[k], cidx(0, 2), w0(o.qw[k], b[0])));
+    T oo = mul(o.vab[k], cidx(1, 1));
+    if constexpr (NC == 15) {
+      ee = add(o.va2b2[k], cidx(2, 2), add(o.va4[k], cidx(4, 0), add(o.vb4[k], cidx(0, 4), ee)));
+      oo = add(o.va3b[k], cidx(3, 1), add(o.vab3[k], cidx(1, 3), oo));
+    }
+    const T oe = add(o.va3[k], cidx(3, 0), add(o.vab2[k], cidx(1, 2), mul(o.va1[k], cidx(1, 0))));
+    const T eo = add(o.vb3[k], cidx(0, 3), add(o.va2b[k], cidx(2, 1), mul(o.vb1[k], cidx(0, 1))));
+    const T s1 = ee + oo, s2 = ee - oo, t1 = oe + eo, t2 = oe - eo;
+    v.pp[k] = s1 + t1;
+    v.mm[k] = s1 - t1;
+    v.pm[k] = s2 + t2;
+    v.mp[k] = s2 - t2;
+  }
+}
+
+// The constants of h37::to_polynomial (FP64) and of its correctly rounded form for
+// the rule's c.
+struct HMap {
+  double v[13];
+  __device__ __forceinline__ double ns() const { return v[0]; }
+  __device__ __forceinline__ double ns3() const { return v[1]; }
+  __device__ __forceinline__ double ns6() const { return v[2]; }
+  __device__ __forceinline__ double s2() const { return v[3]; }
+  __device__ __forceinline__ double s2x3() const { return v[4]; }
+  __device__ __forceinline__ double n1() const { return v[5]; }
+  __device__ __forceinline__ double n2() const { return v[6]; }
+  __device__ __forceinline__ double n2h() const { return v[7]; }
+  __device__ __forceinline__ double n3h() const { return v[8]; }
+  __device__ __forceinline__ double n3s() const { return v[9]; }
+  __device__ __forceinline__ double n4q() const { return v[10]; }
+  __device__ __forceinline__ double n4s() const { return v[11]; }
+  __device__ __forceinline__ double n4f() const { return v[12]; }
+};
+struct HSplitMap {
+  h37::Split v[h37::kMapTerms];
+  __device__ __forceinline__ h37::Split at(int t) const { return v[t]; }
+};
+template <typename T, int NA, int NQ>
+struct HSplitWeights {
+  h37::Split w0, pw[NA], qw[NQ];
+};
+template <typename T, int NA, int NQ>
+struct OrbitRule;
+template <int NA, int NQ>
+struct OrbitRule<double, NA, NQ> {
+  Orbits<double, NA, NQ> o;
+  HMap map;
+};
+template <int NA, int NQ>
+struct OrbitRule<float, NA, NQ> {
+  Orbits<float, NA, NQ> o;
+  HSplitMap map;
+  HSplitWeights<float, NA, NQ> w;
+};
+
+// sums of |e_x^p e_y^q| over any 37 velocities with |e| <= 3 (p + q = 4: at most
+// 36 * 81), and over p + q <= 4 at (3, 3) (547), as powers of two
+constexpr int kOrbitMomentBits = 12;
+constexpr int kOrbitPolynomialBits = 10;
+
+template <int NA, int NQ, int NC>
+__device__ __forceinline__ bool orbit_update(const OrbitRule<double, NA, NQ>& rule, OrbitValues<double, NA, NQ>& v,
+                                             const h37::MomentModel<double>& m) {
+  double M[NC], H[NC], inc[NC];
+  orbit_moments<double>(rule.o, v, M);
+  h37::to_basis<double, NC>(M, H, m);
+  const bool ok = h37::moment_increments<double, NC>(H, inc, m);
+#pragma unroll
+  for (int k = 3; k < NC; ++k) M[k] += inc[k];
+  h37::to_polynomial<double, NC>(M, rule.map);
+  orbit_values<double>(rule.o, M, v, true);
+  return ok;
+}
+
+// FP32, correctly rounded (see h37_moments.cuh)
+template <int NA, int NQ, int NC>
+__device__ __forceinline__ bool orbit_update(const OrbitRule<float, NA, NQ>& rule, OrbitValues<float, NA, NQ>& v,
+                                             const h37::MomentModel<float>& m) {
+  float mx = 0.f;
+  v.each(rule.o, [&](float& x, int, int, int, int) { mx = fmaxf(mx, fabsf(x)); });
+  const float sigma = h37::cut_at(mx, kOrbitMomentBits);
+  OrbitValues<f2, NA, NQ> x;
+  x.r = h37::cut(v.r, sigma);
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    x.xp[k] = h37::cut(v.xp[k], sigma);
+    x.xm[k] = h37::cut(v.xm[k], sigma);
+    x.yp[k] = h37::cut(v.yp[k], sigma);
+    x.ym[k] = h37::cut(v.ym[k], sigma);
+  }
+#pragma unroll
+  for (int k = 0; k < NQ; ++k) {
+    x.pp[k] = h37::cut(v.pp[k], sigma);
+    x.mp[k] = h37::cut(v.mp[k], sigma);
+    x.pm[k] = h37::cut(v.pm[k], sigma);
+    x.mm[k] = h37::cut(v.mm[k], sigma);
+  }
+  f2 M2[NC];
+  orbit_moments<f2>(rule.o, x, M2);
+  float M[NC], L[NC], H[NC], inc[NC], s[NC], c[NC];
+  h37::round_parts<NC>(M2, M, L);
+  h37::to_basis_exact<NC>(M, L, H, m);
+  const bool ok = h37::moment_increments<float, NC>(H, inc, m);
+  h37::add_increments<NC>(M, L, inc);
+  h37::to_polynomial_exact<NC>(M, L, rule.map, s, c);
+  f2 b[NC];
+  h37::cut_polynomial<NC>(s, c, b, kOrbitPolynomialBits);
+  orbit_values<f2>(rule.o, b, x, false);
+  v.r = h37::weigh(x.r, rule.w.w0);
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    v.xp[k] = h37::weigh(x.xp[k], rule.w.pw[k]);
+    v.xm[k] = h37::weigh(x.xm[k], rule.w.pw[k]);
+    v.yp[k] = h37::weigh(x.yp[k], rule.w.pw[k]);
+    v.ym[k] = h37::weigh(x.ym[k], rule.w.pw[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < NQ; ++k) {
+    v.pp[k] = h37::weigh(x.pp[k], rule.w.qw[k]);
+    v.mp[k] = h37::weigh(x.mp[k], rule.w.qw[k]);
+    v.pm[k] = h37::weigh(x.pm[k], rule.w.qw[k]);
+    v.mm[k] = h37::weigh(x.mm[k], rule.w.qw[k]);
+  }
+  return ok;
+}
+
+// The sweep of hgen_sweep_kernel by orbits, threads walking the nodes in one dimension.
+template <typename T, int NC, int NA, int NQ, bool ODD>
+__global__ void __launch_bounds__(kHgThreads)
+    hgen_orbit_kernel(T* __restrict__ f, HGrid g, const __grid_constant__ OrbitRule<T, NA, NQ> rule,
+                      const __grid_constant__ h37::MomentModel<T> m, int* __restrict__ status) {
+  const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
+  if (node >= (uint32_t)g.N) return;
+  const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
+  OrbitValues<T, NA, NQ> v;
+  v.each(rule.o, [&](T& val, int i, int ex, int ey, int opp) {
+    val = ODD ? f[(size_t)opp * g.N + hnbr(g, x, y, -ex, -ey)] : f[(size_t)i * g.N + node];
+  });
+  if (!orbit_update<NA, NQ, NC>(rule, v, m)) atomicOr(status, 1);
+  v.each(rule.o, [&](T& val, int i, int ex, int ey, int opp) {
+    if (ODD)
+      f[(size_t)i * g.N + hnbr(g, x, y, ex, ey)] = val;
+    else
+      f[(size_t)opp * g.N + node] = val;
+  });
+}
+
 __device__ __forceinline__ void hxy_of(const HGrid& g, int64_t n, int& x, int& y) {
   const uint32_t nn = (uint32_t)n, nx = (uint32_t)g.nx;
   y = (int)(nn / nx);
@@ -379,6 +735,70 @@ inline h37::Model hmodel(const Sim* s) {
   return m;
 }
 
+void fill_map(double c2, int, HMap* k) {
+  const double s = 1.0 / c2, n = c2;
+  const double v[13] = {-s, -3.0 * s, -6.0 * s, s * s, 3.0 * s * s, n, n * n, 0.5 * n * n, 0.5 * n * n * n,
+                        n * n * n / 6.0, 0.25 * n * n * n * n, n * n * n * n / 6.0, n * n * n * n / 24.0};
+  for (int i = 0; i < 13; ++i) k->v[i] = v[i];
+}
+void fill_map(double c2, int nc, HSplitMap* k) {
+  for (int t = 0; t < h37::kMapTerms; ++t) k->v[t] = h37::split_of(h37::map_term(t, nc, c2));
+}
+template <int NA, int NQ>
+bool fill_rule(const HLattice& L, int nc, OrbitRule<double, NA, NQ>* r) {
+  fill_map(L.c * L.c, nc, &r->map);
+  return make_orbits(L, true, &r->o);
+}
+template <int NA, int NQ>
+bool fill_rule(const HLattice& L, int nc, OrbitRule<float, NA, NQ>* r) {
+  fill_map(L.c * L.c, nc, &r->map);
+  if (!make_orbits(L, false, &r->o)) return false;
+  r->w.w0 = h37::split_of(L.w[r->o.rest]);
+  for (int k = 0; k < NA; ++k) r->w.pw[k] = h37::split_of(L.w[r->o.xp[k]]);
+  for (int k = 0; k < NQ; ++k) r->w.qw[k] = h37::split_of(L.w[r->o.pp[k]]);
+  return true;
+}
+
+template <typename T>
+h37::MomentModel<T> hmoment_model(const Sim* s) {
+  h37::MomentModel<T> m;
+  const double sl = 1.0 / (s->hl.c * s->hl.c), tau = h37::basis_temperature(s->theta_ref * sl);
+  for (int n = 0; n < 5; ++n) m.no[n] = (T)-s->rates.w[n];
+  m.s = (T)sl;
+  m.basis = (T)tau;
+  m.basis2x3 = (T)(3.0 * tau * tau);
+  m.th_ref = (T)(s->theta_ref * sl - tau);
+  m.th_iso = (T)(sl - tau);
+  m.kext = 0;
+  m.usq_max = (T)(4.0 * sl);
+  m.thermal = (s->flags & LBM_THERMAL) ? 1 : 0;
+  m.raw = 0;
+  m.sround = 0;
+  m.seed = 0;
+  return m;
+}
+
+// The orbit sweep if the rule has NA and NQ orbits of each kind; *taken says so.
+template <int S, int NC, int NA, int NQ>
+cudaError_t orbit_sweep(Sim* s, int odd, bool* taken) {
+  using T = typename HStore<S>::type;
+  OrbitRule<T, NA, NQ> rule;
+  *taken = fill_rule(s->hl, NC, &rule);
+  if (!*taken) return cudaSuccess;
+  // the largest of 128, 64, 32 threads that gives every SM two blocks: small grids spread over all of them
+  int t = kHgThreads;
+  while (t > 32 && s->N < (int64_t)t * 2 * 152) t /= 2;
+  const unsigned blocks = (unsigned)((s->N + t - 1) / t);
+  T* f = static_cast<T*>(s->pop);
+  if (odd)
+    hgen_orbit_kernel<T, NC, NA, NQ, true><<<blocks, t, 0, s->stream>>>(f, hgrid(s), rule, hmoment_model<T>(s),
+                                                                        status_word(s));
+  else
+    hgen_orbit_kernel<T, NC, NA, NQ, false><<<blocks, t, 0, s->stream>>>(f, hgrid(s), rule, hmoment_model<T>(s),
+                                                                         status_word(s));
+  return cudaGetLastError();
+}
+
 template <int S, int Q, int NC, bool EXACT>
 cudaError_t sweep_e(Sim* s, int odd, const HSplit& sp) {
   using E = typename HStore<S>::type;
@@ -396,6 +816,20 @@ cudaError_t sweep_e(Sim* s, int odd, const HSplit& sp) {
 // FP32 storage takes the correctly rounded transforms unless LBM_FAST_TRANSFORMS.
 template <int S, int Q, int NC>
 cudaError_t sweep_t(Sim* s, int odd) {
+  if (S == LBM_F64 || !(s->flags & LBM_FAST_TRANSFORMS)) {
+    // the orbit counts of the minimal rules: 37 velocities have three axis shells, 17 one or two
+    bool taken = false;
+    cudaError_t e;
+    if constexpr (Q == 37) {
+      e = orbit_sweep<S, NC, 3, 6>(s, odd, &taken);
+      if (taken) return e;
+    } else {
+      e = orbit_sweep<S, NC, 2, 2>(s, odd, &taken);
+      if (taken) return e;
+      e = orbit_sweep<S, NC, 1, 3>(s, odd, &taken);
+      if (taken) return e;
+    }
+  }
   // host staging of the split tables, one per host thread (the launch copies its parameters)
   thread_local static HSplit sp;
   if constexpr (S == LBM_F32) {
