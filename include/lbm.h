@@ -263,8 +263,10 @@ int lbm_set_active_planes(lbm_handle h, int64_t z_lo, int64_t z_count);
  * current settings (environment switches included), for example
  * "tp_pair_kernel" (two nodes per thread), "tp_pair_zrun_kernel" (the same
  * walking several planes per thread: D3Q27 with FP16 / BF16 offsets),
- * "tp_sweep_kernel" (one node per thread), "h37_pair_kernel", "learned_tc_kernel".  Measurement and tests only;
- * the string is static.  NULL for a NULL handle (no error code). */
+ * "tp_sweep_kernel" (one node per thread), "tp_column_kernel" (two nodes of a
+ * column per thread: odd nx), "h37_pair_kernel", "learned_tc_kernel".  A call of
+ * several steps on an FP32 grid larger than L2 may run them in one launch of the
+ * same arithmetic.  Measurement and tests only; the string is static.  NULL for a NULL handle (no error code). */
 const char* lbm_sweep_kernel(lbm_handle h);
 
 /* Failure-detection self-test.  The paper has no counterpart; it exercises the

@@ -11,6 +11,7 @@
 
 #include "h37_moments.cuh"
 #include "pair_io.cuh"
+#include "pdl.cuh"
 #include "reduce.cuh"
 
 namespace lbm {
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(kH37Threads)
   using T = typename h37::Store<S>::calc;
   constexpr bool kScaled = S == LBM_F16 || S == LBM_BF16;
   const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_wait();
   if (node >= (uint32_t)g.N) return;
   const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
   T v[h37::kQ];
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
     h37_pair_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, SweepModel<S, false> m,
                     int* __restrict__ status) {
   const int xp = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_wait();
   if (2 * xp >= g.nx) return;
   h37_pair_update<S, ODD, false>(f, g, m, status, xp, nullptr);
 }
@@ -275,6 +278,7 @@ __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
                            int* __restrict__ status, float* __restrict__ partials) {
   const int xp = blockIdx.x * blockDim.x + threadIdx.x;
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  chain_wait();
   if (2 * xp < g.nx) {
     f2 mom[3];
     h37_pair_update<S, ODD, true>(f, g, m, status, xp, mom);
@@ -467,11 +471,8 @@ cudaError_t pair_t(Sim* s, int odd) {
   using E = typename PairIO<S>::E;
   dim3 grid((unsigned)((s->nx / 2 + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
   E* f = static_cast<E*>(s->pop);
-  if (odd)
-    h37_pair_kernel<S, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s));
-  else
-    h37_pair_kernel<S, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s));
-  return cudaGetLastError();
+  return launch_chained(odd ? h37_pair_kernel<S, true> : h37_pair_kernel<S, false>, grid, dim3(kH37Threads), s->stream, f,
+                        grid2(s), sweep_model<S, false>(s), status_word(s));
 }
 
 template <int S>
@@ -479,11 +480,8 @@ cudaError_t pair_totals_t(Sim* s, int odd, float* partials) {
   using E = typename PairIO<S>::E;
   dim3 grid((unsigned)((s->nx / 2 + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
   E* f = static_cast<E*>(s->pop);
-  if (odd)
-    h37_pair_totals_kernel<S, true><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s), partials);
-  else
-    h37_pair_totals_kernel<S, false><<<grid, kH37Threads, 0, s->stream>>>(f, grid2(s), sweep_model<S, false>(s), status_word(s), partials);
-  return cudaGetLastError();
+  return launch_chained(odd ? h37_pair_totals_kernel<S, true> : h37_pair_totals_kernel<S, false>, grid, dim3(kH37Threads),
+                        s->stream, f, grid2(s), sweep_model<S, false>(s), status_word(s), partials);
 }
 
 // Threads per block of the one-node sweep: the largest of 128, 64, 32 that gives
@@ -504,9 +502,8 @@ cudaError_t sweep_t(Sim* s, int odd) {
   const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   E* f = static_cast<E*>(s->pop);
   auto launch = [&](auto odd_c, auto exact_c) {
-    h37_sweep_kernel<S, decltype(odd_c)::value, decltype(exact_c)::value>
-        <<<blocks, t, 0, s->stream>>>(f, grid2(s), sweep_model<S, decltype(exact_c)::value>(s), status_word(s));
-    return cudaGetLastError();
+    return launch_chained(h37_sweep_kernel<S, decltype(odd_c)::value, decltype(exact_c)::value>, dim3(blocks), dim3(t),
+                          s->stream, f, grid2(s), sweep_model<S, decltype(exact_c)::value>(s), status_word(s));
   };
   if constexpr (S == LBM_F32) {
     if (h37_exact_transforms(s))

@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "h37_moments.cuh"
+#include "pdl.cuh"
 #include "reduce.cuh"
 
 namespace lbm {
@@ -540,25 +541,39 @@ __device__ __forceinline__ bool orbit_update(const OrbitRule<float, NA, NQ>& rul
   return ok;
 }
 
-// The sweep of hgen_sweep_kernel by orbits, threads walking the nodes in one dimension.
-template <typename T, int NC, int NA, int NQ, bool ODD>
-__global__ void __launch_bounds__(kHgThreads)
-    hgen_orbit_kernel(T* __restrict__ f, HGrid g, const __grid_constant__ OrbitRule<T, NA, NQ> rule,
-                      const __grid_constant__ h37::MomentModel<T> m, int* __restrict__ status) {
-  const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
-  if (node >= (uint32_t)g.N) return;
-  const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
-  OrbitValues<T, NA, NQ> v;
+template <bool ODD, typename T, int NA, int NQ>
+__device__ __forceinline__ void orbit_load(const T* __restrict__ f, const HGrid& g, const OrbitRule<T, NA, NQ>& rule,
+                                           int x, int y, OrbitValues<T, NA, NQ>& v) {
+  const uint32_t node = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
   v.each(rule.o, [&](T& val, int i, int ex, int ey, int opp) {
     val = ODD ? f[(size_t)opp * g.N + hnbr(g, x, y, -ex, -ey)] : f[(size_t)i * g.N + node];
   });
-  if (!orbit_update<NA, NQ, NC>(rule, v, m)) atomicOr(status, 1);
+}
+template <bool ODD, typename T, int NA, int NQ>
+__device__ __forceinline__ void orbit_store(T* __restrict__ f, const HGrid& g, const OrbitRule<T, NA, NQ>& rule, int x,
+                                            int y, OrbitValues<T, NA, NQ>& v) {
+  const uint32_t node = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
   v.each(rule.o, [&](T& val, int i, int ex, int ey, int opp) {
     if (ODD)
       f[(size_t)i * g.N + hnbr(g, x, y, ex, ey)] = val;
     else
       f[(size_t)opp * g.N + node] = val;
   });
+}
+
+// The sweep of hgen_sweep_kernel by orbits, threads walking the nodes in one dimension.
+template <typename T, int NC, int NA, int NQ, bool ODD>
+__global__ void __launch_bounds__(kHgThreads)
+    hgen_orbit_kernel(T* __restrict__ f, HGrid g, const __grid_constant__ OrbitRule<T, NA, NQ> rule,
+                      const __grid_constant__ h37::MomentModel<T> m, int* __restrict__ status) {
+  const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_wait();
+  if (node >= (uint32_t)g.N) return;
+  const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
+  OrbitValues<T, NA, NQ> v;
+  orbit_load<ODD>(f, g, rule, x, y, v);
+  if (!orbit_update<NA, NQ, NC>(rule, v, m)) atomicOr(status, 1);
+  orbit_store<ODD>(f, g, rule, x, y, v);
 }
 
 __device__ __forceinline__ void hxy_of(const HGrid& g, int64_t n, int& x, int& y) {
@@ -790,13 +805,8 @@ cudaError_t orbit_sweep(Sim* s, int odd, bool* taken) {
   while (t > 32 && s->N < (int64_t)t * 2 * 152) t /= 2;
   const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   T* f = static_cast<T*>(s->pop);
-  if (odd)
-    hgen_orbit_kernel<T, NC, NA, NQ, true><<<blocks, t, 0, s->stream>>>(f, hgrid(s), rule, hmoment_model<T>(s),
-                                                                        status_word(s));
-  else
-    hgen_orbit_kernel<T, NC, NA, NQ, false><<<blocks, t, 0, s->stream>>>(f, hgrid(s), rule, hmoment_model<T>(s),
-                                                                         status_word(s));
-  return cudaGetLastError();
+  return launch_chained(odd ? hgen_orbit_kernel<T, NC, NA, NQ, true> : hgen_orbit_kernel<T, NC, NA, NQ, false>,
+                        dim3(blocks), dim3(t), s->stream, f, hgrid(s), rule, hmoment_model<T>(s), status_word(s));
 }
 
 template <int S, int Q, int NC, bool EXACT>

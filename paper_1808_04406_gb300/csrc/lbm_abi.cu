@@ -17,6 +17,8 @@ namespace lbm {
 bool closure_uses_tcgen05();
 // tp_pair.cu: the kernel tp_launch_pair_sweep launches for this handle.
 const char* tp_pair_kernel_name(const Sim* s);
+// tp_sweep.cu: that of tp_launch_sweep.
+const char* tp_sweep_kernel_name(const Sim* s);
 
 static thread_local char g_err[512] = "";
 
@@ -736,7 +738,7 @@ const char* lbm_sweep_kernel(lbm_handle h) {
   if (is_hgen(s)) return "hgen_sweep_kernel";
   if (is_h37(s)) return h37_pair_supported(s) ? "h37_pair_kernel" : "h37_sweep_kernel";
   if (s->closure) return closure_uses_tcgen05() ? "learned_tc_kernel" : "learned_sweep_kernel";
-  return tp_pair_supported(s) ? tp_pair_kernel_name(s) : "tp_sweep_kernel";
+  return tp_pair_supported(s) ? tp_pair_kernel_name(s) : tp_sweep_kernel_name(s);
 }
 
 int lbm_selftest_wait_timeout(lbm_handle h, int polls) {

@@ -18,6 +18,8 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "flat_index.cuh"
+#include "pdl.cuh"
 #include "sweep_body.cuh"
 
 namespace lbm {
@@ -26,22 +28,31 @@ namespace {
 #ifndef LBM_PAIR_THREADS
 #define LBM_PAIR_THREADS 128
 #endif
-#ifndef LBM_PAIR_MINB
-#define LBM_PAIR_MINB 3
-#endif
 constexpr int kPairThreads = LBM_PAIR_THREADS;
+// Blocks per SM: with the stores' addresses computed anew instead of kept from the
+// loads (54 registers on D3Q27) the sweeps take 128 registers or less.
+constexpr int kPairMinBlocks = 4;
+
+// The compiler does not know these values to be what they were.
+__device__ __forceinline__ void forget(int& x, int& y, int& z) { asm volatile("" : "+r"(x), "+r"(y), "+r"(z)); }
 
 template <int D, int S, bool ODD>
-__global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MINB)
+__global__ void __launch_bounds__(kPairThreads, kPairMinBlocks)
     tp_pair_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r,
-                   int* __restrict__ status, int z0) {
-  const int xp = blockIdx.x * blockDim.x + threadIdx.x;
-  if (xp >= (g.nx >> 1)) return;
-  const int y = blockIdx.y, z = blockIdx.z + z0;  // z0: first plane of the swept range
+                   int* __restrict__ status, RowLength row, int z0) {
+  int xp, y;
+  const bool in = row_of(blockIdx.x * blockDim.x + threadIdx.x, row, g.ny, xp, y);
+  int z = blockIdx.z + z0;  // z0: first plane of the swept range
+  chain_wait();
+  if (!in) return;
   f2 om[2 * D + 1];
 #pragma unroll
   for (int n = 0; n <= 2 * D; ++n) om[n] = cst<f2>(r.w[n]);
-  if (!tp::update_pair<D, S, ODD>(f, g, om, xp, y, z)) atomicOr(status, 1);
+  f2 v[tp::qof<D>()];
+  tp::pair_load<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
+  if constexpr (D == 3) forget(xp, y, z);
+  if (!tp::collide<f2, D>(v, om)) atomicOr(status, 1);
+  tp::pair_store<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
 }
 
 // The same sweep for D3Q27 with 16-bit offsets, each thread walking kZRun
@@ -53,17 +64,24 @@ __global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MINB)
 // tp_pair_kernel, and so are the results, bit for bit.  At 4 blocks per SM the
 // compiler keeps it within 128 registers without spills (the one-pair kernel
 // needs 158-164 and so runs at 3).
+//
+// The walk is 8 planes, or fewer where that would leave less than 900 blocks, one
+// and a half waves of 608 (FP16, us a step, walks of 8 and of 1: 64^3 10.9 and 7.7,
+// 96^3 28.5 and 21.2, 128^3 with 1024 blocks 49.8 and 51.9, 256^3 356 and 401).
 constexpr int kZRun = 8;
 constexpr int kZRunMinBlocks = 4;
+constexpr int kZRunMinGrid = 900;
 
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kPairThreads, kZRunMinBlocks)
     tp_pair_zrun_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r, int* __restrict__ status,
-                        int z0, int z1) {
-  const int xp = blockIdx.x * blockDim.x + threadIdx.x;
-  if (xp >= (g.nx >> 1)) return;
-  const int y = blockIdx.y, zb = z0 + (int)blockIdx.z * kZRun;
-  const int ze = zb + kZRun < z1 ? zb + kZRun : z1;  // planes zb .. ze - 1
+                        RowLength row, int z0, int z1, int run) {
+  int xp, y;
+  const bool in = row_of(blockIdx.x * blockDim.x + threadIdx.x, row, g.ny, xp, y);
+  chain_wait();
+  if (!in) return;
+  const int zb = z0 + (int)blockIdx.z * run;
+  const int ze = zb + run < z1 ? zb + run : z1;  // planes zb .. ze - 1
   f2 om[7];
 #pragma unroll
   for (int n = 0; n < 7; ++n) om[n] = cst<f2>(r.w[n]);
@@ -75,7 +93,9 @@ __global__ void __launch_bounds__(kPairThreads, kZRunMinBlocks)
     tp::pair_decode<3, S, ODD>(raw, v);
     if (z + 1 < ze) tp::pair_load_raw<3, S, ODD>(f, g, tp::PairAddr<3, ODD>(g, xp, y, z + 1), raw);
     ok = tp::collide<f2, 3>(v, om) && ok;
-    tp::pair_store<3, S, ODD>(f, g, tp::PairAddr<3, ODD>(g, xp, y, z), v);
+    int zs = z;
+    forget(xp, y, zs);
+    tp::pair_store<3, S, ODD>(f, g, tp::PairAddr<3, ODD>(g, xp, y, zs), v);
   }
   if (!ok) atomicOr(status, 1);
 }
@@ -87,12 +107,15 @@ __global__ void __launch_bounds__(kPairThreads, kZRunMinBlocks)
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kPairThreads, 3)  // the running totals need more than 128 registers
     tp_pair_zrun_totals_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r,
-                               int* __restrict__ status, float* __restrict__ partials, int z0, int z1) {
-  const int xp = blockIdx.x * blockDim.x + threadIdx.x;
+                               int* __restrict__ status, float* __restrict__ partials, RowLength row, int z0,
+                               int z1, int run) {
+  int xp, y;
+  const bool in = row_of(blockIdx.x * blockDim.x + threadIdx.x, row, g.ny, xp, y);
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  if (xp < (g.nx >> 1)) {
-    const int y = blockIdx.y, zb = z0 + (int)blockIdx.z * kZRun;
-    const int ze = zb + kZRun < z1 ? zb + kZRun : z1;
+  chain_wait();
+  if (in) {
+    const int zb = z0 + (int)blockIdx.z * run;
+    const int ze = zb + run < z1 ? zb + run : z1;
     f2 om[7];
 #pragma unroll
     for (int n = 0; n < 7; ++n) om[n] = cst<f2>(r.w[n]);
@@ -142,36 +165,47 @@ __global__ void __launch_bounds__(kPairThreads, 3)  // the running totals need m
 // FP64 afterwards.  (FP64 arithmetic runs at a small fraction of the FP32 rate on
 // this GPU: per-node FP64 sums would double the sweep's time; and no block
 // barrier holds finished warps back.)
+//
+// On D3Q27 a thread adds up the pairs of up to kTotalsRun planes first: fewer
+// shuffles (a seventh of the kernel's instructions with one plane) and fewer
+// partials.
+constexpr int kTotalsRun = 4;
 template <int D, int S, bool ODD>
-__global__ void __launch_bounds__(kPairThreads, LBM_PAIR_MINB)
+__global__ void __launch_bounds__(kPairThreads, kPairMinBlocks)
     tp_pair_totals_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r, int* __restrict__ status,
-                          float* __restrict__ partials, int z0) {
-  const int xp = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y, z = blockIdx.z + z0;
+                          float* __restrict__ partials, RowLength row, int z0, int z1, int run) {
+  int xp, y;
+  const bool in = row_of(blockIdx.x * blockDim.x + threadIdx.x, row, g.ny, xp, y);
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  if (xp < (g.nx >> 1)) {
+  chain_wait();
+  if (in) {
     f2 om[2 * D + 1];
 #pragma unroll
     for (int n = 0; n <= 2 * D; ++n) om[n] = cst<f2>(r.w[n]);
-    const tp::PairAddr<D, ODD> A(g, xp, y, z);
-    f2 v[tp::qof<D>()];
-    tp::pair_load<D, S, ODD>(f, g, A, v);
-    tp::NodeMoments<f2, D> m;
-    const bool ok = tp::collide<f2, D, true>(v, om, &m);
-    tp::pair_store<D, S, ODD>(f, g, A, v);
-    if (!ok) atomicOr(status, 1);
-    float d0, d1, jj0 = 0.0f, jj1 = 0.0f;
-    unpack2(m.drho, d0, d1);
-    acc[0] = d0 + d1;
+    const int zb = z0 + (int)blockIdx.z * run, ze = zb + run < z1 ? zb + run : z1;
+    bool ok = true;
+#pragma unroll 1
+    for (int z = zb; z < ze; ++z) {
+      f2 v[tp::qof<D>()];
+      tp::pair_load<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
+      if constexpr (D == 3) forget(xp, y, z);
+      tp::NodeMoments<f2, D> m;
+      ok = tp::collide<f2, D, true>(v, om, &m) && ok;
+      tp::pair_store<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
+      float d0, d1, jj0 = 0.0f, jj1 = 0.0f;
+      unpack2(m.drho, d0, d1);
+      acc[0] += d0 + d1;
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      float j0, j1;
-      unpack2(m.j[d], j0, j1);
-      acc[1 + d] = j0 + j1;
-      jj0 += j0 * j0;
-      jj1 += j1 * j1;
+      for (int d = 0; d < D; ++d) {
+        float j0, j1;
+        unpack2(m.j[d], j0, j1);
+        acc[1 + d] += j0 + j1;
+        jj0 += j0 * j0;
+        jj1 += j1 * j1;
+      }
+      acc[4] += __fdividef(0.5f * jj0, 1.0f + d0) + __fdividef(0.5f * jj1, 1.0f + d1);
     }
-    acc[4] = __fdividef(0.5f * jj0, 1.0f + d0) + __fdividef(0.5f * jj1, 1.0f + d1);
+    if (!ok) atomicOr(status, 1);
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -193,20 +227,28 @@ bool zrun_enabled() {
   return !(e && std::strcmp(e, "0") == 0);
 }
 
+inline unsigned plane_blocks(const Sim* s) {
+  return (unsigned)((s->nx / 2 * s->ny + kPairThreads - 1) / kPairThreads);
+}
+
+// Planes per thread, at most `longest`.
+inline int walk_of(const Sim* s, int longest) {
+  int run = longest;
+  while (run > 1 && (int64_t)plane_blocks(s) * ((active_nz(s) + run - 1) / run) < kZRunMinGrid) run /= 2;
+  return run;
+}
+
 template <int S>
 cudaError_t launch_zrun(Sim* s, int odd) {
   using E = typename PairIO<S>::E;
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
-  const int64_t pairs = s->nx / 2, nzs = active_nz(s);
-  dim3 grid((unsigned)((pairs + kPairThreads - 1) / kPairThreads), (unsigned)s->ny,
-            (unsigned)((nzs + kZRun - 1) / kZRun));
+  const int64_t nzs = active_nz(s);
+  const int run = walk_of(s, kZRun);
+  dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
   const int z0 = (int)active_z0(s), z1 = (int)(active_z0(s) + nzs);
   E* f = static_cast<E*>(s->pop);
-  if (odd)
-    tp_pair_zrun_kernel<S, true><<<grid, kPairThreads, 0, s->stream>>>(f, g, s->rates, status_word(s), z0, z1);
-  else
-    tp_pair_zrun_kernel<S, false><<<grid, kPairThreads, 0, s->stream>>>(f, g, s->rates, status_word(s), z0, z1);
-  return cudaGetLastError();
+  return launch_chained(odd ? tp_pair_zrun_kernel<S, true> : tp_pair_zrun_kernel<S, false>, grid, dim3(kPairThreads),
+                        s->stream, f, g, s->rates, status_word(s), row_length(s->nx / 2), z0, z1, run);
 }
 
 template <int D, int S>
@@ -216,34 +258,25 @@ cudaError_t launch(Sim* s, int odd) {
     if (zrun_enabled()) return launch_zrun<S>(s, odd);
   }
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
-  const int64_t pairs = s->nx / 2;
   dim3 block(kPairThreads);
-  dim3 grid((unsigned)((pairs + kPairThreads - 1) / kPairThreads), (unsigned)s->ny, (unsigned)active_nz(s));
+  dim3 grid(plane_blocks(s), 1, (unsigned)active_nz(s));
   const int z0 = (int)active_z0(s);
   E* f = static_cast<E*>(s->pop);
-  if (odd)
-    tp_pair_kernel<D, S, true><<<grid, block, 0, s->stream>>>(f, g, s->rates, status_word(s), z0);
-  else
-    tp_pair_kernel<D, S, false><<<grid, block, 0, s->stream>>>(f, g, s->rates, status_word(s), z0);
-  return cudaGetLastError();
+  return launch_chained(odd ? tp_pair_kernel<D, S, true> : tp_pair_kernel<D, S, false>, grid, block, s->stream, f, g,
+                        s->rates, status_word(s), row_length(s->nx / 2), z0);
 }
 
 template <int S>
 cudaError_t launch_zrun_totals(Sim* s, int odd, float* partials) {
   using E = typename PairIO<S>::E;
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
-  const int64_t pairs = s->nx / 2, nzs = active_nz(s);
-  dim3 grid((unsigned)((pairs + kPairThreads - 1) / kPairThreads), (unsigned)s->ny,
-            (unsigned)((nzs + kZRun - 1) / kZRun));
+  const int64_t nzs = active_nz(s);
+  const int run = walk_of(s, kZRun);
+  dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
   const int z0 = (int)active_z0(s), z1 = (int)(active_z0(s) + nzs);
   E* f = static_cast<E*>(s->pop);
-  if (odd)
-    tp_pair_zrun_totals_kernel<S, true><<<grid, kPairThreads, 0, s->stream>>>(f, g, s->rates, status_word(s),
-                                                                               partials, z0, z1);
-  else
-    tp_pair_zrun_totals_kernel<S, false><<<grid, kPairThreads, 0, s->stream>>>(f, g, s->rates, status_word(s),
-                                                                                partials, z0, z1);
-  return cudaGetLastError();
+  return launch_chained(odd ? tp_pair_zrun_totals_kernel<S, true> : tp_pair_zrun_totals_kernel<S, false>, grid,
+                        dim3(kPairThreads), s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
 }
 
 template <int D, int S>
@@ -253,16 +286,14 @@ cudaError_t launch_totals(Sim* s, int odd, float* partials) {
     if (zrun_enabled()) return launch_zrun_totals<S>(s, odd, partials);
   }
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
-  const int64_t pairs = s->nx / 2;
+  const int64_t nzs = active_nz(s);
   dim3 block(kPairThreads);
-  dim3 grid((unsigned)((pairs + kPairThreads - 1) / kPairThreads), (unsigned)s->ny, (unsigned)active_nz(s));
-  const int z0 = (int)active_z0(s);
+  const int run = D == 2 ? 1 : walk_of(s, kTotalsRun);
+  dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
+  const int z0 = (int)active_z0(s), z1 = (int)(z0 + nzs);
   E* f = static_cast<E*>(s->pop);
-  if (odd)
-    tp_pair_totals_kernel<D, S, true><<<grid, block, 0, s->stream>>>(f, g, s->rates, status_word(s), partials, z0);
-  else
-    tp_pair_totals_kernel<D, S, false><<<grid, block, 0, s->stream>>>(f, g, s->rates, status_word(s), partials, z0);
-  return cudaGetLastError();
+  return launch_chained(odd ? tp_pair_totals_kernel<D, S, true> : tp_pair_totals_kernel<D, S, false>, grid, block,
+                        s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
 }
 
 template <int D>
@@ -299,8 +330,8 @@ cudaError_t tp_launch_pair_sweep(Sim* s, int odd) {
 
 int64_t tp_pair_warps(const Sim* s) {
   const int64_t nz = active_nz(s);
-  const int64_t planes = s->D == 3 && s->storage != LBM_F32 && zrun_enabled() ? (nz + kZRun - 1) / kZRun : nz;
-  return ((s->nx / 2 + kPairThreads - 1) / kPairThreads) * s->ny * planes * (kPairThreads / 32);
+  const int run = s->D == 2 ? 1 : walk_of(s, s->storage != LBM_F32 && zrun_enabled() ? kZRun : kTotalsRun);
+  return (int64_t)plane_blocks(s) * ((nz + run - 1) / run) * (kPairThreads / 32);
 }
 
 cudaError_t tp_launch_pair_sweep_totals(Sim* s, int odd, float* partials) {
