@@ -108,8 +108,9 @@ typedef struct lbm_sim* lbm_handle;
 #define LBM_ECUDA (-2)     /* a CUDA runtime call failed */
 #define LBM_EDIVERGED (-3) /* a node left the range the collision is defined on (lbm_status) */
 #define LBM_ESIZE (-4)     /* a caller buffer is smaller than lbm_query_bytes asks */
-#define LBM_ETIMEOUT (-5)  /* a bounded device-side wait (tensor-core completion) gave up; the
-                              sweep that saw it skipped its remaining tiles */
+#define LBM_ETIMEOUT (-5)  /* a bounded device-side wait (tensor-core completion, or a tile's
+                              neighbours in a launch of several steps) gave up; the sweep that
+                              saw it skipped its remaining tiles */
 #define LBM_EOOM (-6)      /* a host allocation of the library's own bookkeeping failed */
 
 /* Bytes of the population buffer and of the workspace a simulation needs.

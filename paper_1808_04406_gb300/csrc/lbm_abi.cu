@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 
@@ -19,6 +20,8 @@ bool closure_uses_tcgen05();
 const char* tp_pair_kernel_name(const Sim* s);
 // tp_sweep.cu: that of tp_launch_sweep.
 const char* tp_sweep_kernel_name(const Sim* s);
+// tp_multi.cu: up to n steps in one launch; *done = steps taken (0: one sweep at a time only).
+cudaError_t tp_launch_steps(Sim* s, int64_t n, int* done);
 
 static thread_local char g_err[512] = "";
 
@@ -120,7 +123,7 @@ int sync_and_status(Sim* s, int rc) {
   if (e) return e;
   e = cuda_check(cudaStreamSynchronize(s->stream), "stream synchronize");
   if (e) return e;
-  if (st & 2) return set_error(LBM_ETIMEOUT, "a bounded device wait for tensor-core completion gave up");
+  if (st & 2) return set_error(LBM_ETIMEOUT, "a bounded device wait (tensor-core completion, or the neighbours of a tile) gave up");
   if (st) return set_error(LBM_EDIVERGED, "a node diverged (rho <= 0, |u| >= 1 or non-finite)");
   return LBM_OK;
 }
@@ -212,10 +215,35 @@ cudaError_t launch_sweep(Sim* s) {
   return tp_pair_supported(s) ? tp_launch_pair_sweep(s, odd) : tp_launch_sweep(s, odd);
 }
 
+// up to n steps in one launch; *done = 0 where only single sweeps are possible
+cudaError_t launch_steps(Sim* s, int64_t n, int* done) {
+  *done = 0;
+  // LBM_MULTI_STEP=0 keeps one launch per step (read at every call; used to compare the two)
+  const char* e = std::getenv("LBM_MULTI_STEP");
+  if (n < 2 || s->closure || s->z_cnt > 0 || (e && std::strcmp(e, "0") == 0)) return cudaSuccess;
+  return hermite_family(s) ? cudaSuccess : tp_launch_steps(s, n, done);
+}
+
 cudaError_t launch_reduce_into(Sim* s, double* partials, int nblocks, double* result) {
   if (is_hgen(s)) return hgen_launch_reduce_into(s, partials, nblocks, result);
   return is_h37(s) ? h37_launch_reduce_into(s, partials, nblocks, result)
                    : tp_launch_reduce_into(s, partials, nblocks, result);
+}
+
+// n steps, several per launch where that is possible
+static int advance(Sim* s, int64_t n) {
+  while (n > 0) {
+    int done = 0;
+    cudaError_t e = launch_steps(s, n, &done);
+    if (e == cudaSuccess && done < 1) {
+      e = launch_sweep(s);
+      done = 1;
+    }
+    if (e != cudaSuccess) return cuda_check(e, "sweep kernel");
+    s->step += done;
+    n -= done;
+  }
+  return LBM_OK;
 }
 
 }  // namespace lbm
@@ -475,12 +503,7 @@ int lbm_step(lbm_handle h, int64_t n) {
   Sim* s = as_sim(h);
   if (int rc = check_handle(s)) return rc;
   if (n < 0) return set_error(LBM_EINVAL, "negative step count");
-  for (int64_t k = 0; k < n; ++k) {
-    cudaError_t e = launch_sweep(s);
-    if (e != cudaSuccess) return cuda_check(e, "sweep kernel");
-    ++s->step;
-  }
-  return LBM_OK;
+  return advance(s, n);
 }
 
 int lbm_moments(lbm_handle h, void* rho, void* u, void* theta, int dtype, int on_device) {
@@ -682,12 +705,7 @@ int lbm_mode_history(lbm_handle h, int field, const int64_t mode[3], int n_recor
   double* hist = history_buf(s);
   int rc = LBM_OK;
   for (int r = 0; r < n_records && !rc; ++r) {
-    if (r > 0) {
-      for (int64_t k = 0; k < stride && !rc; ++k) {
-        rc = cuda_check(launch_sweep(s), "sweep kernel");
-        if (!rc) ++s->step;
-      }
-    }
+    if (r > 0) rc = advance(s, stride);
     if (!rc) rc = cuda_check(launch_mode_into(s, field, mode, hist + 2 * r), "mode amplitude kernels");
   }
   // the density amplitude is accumulated from rho - 1; restore sum_x 1 at k = 0
