@@ -23,6 +23,7 @@
 
 #include "lbm_internal.cuh"
 #include "mlp.cuh"
+#include "pdl.cuh"
 #include "sweep_body.cuh"
 #include "tc05.cuh"
 #include "tp_common.cuh"
@@ -183,19 +184,26 @@ __global__ void rescale_kernel(float* __restrict__ f, int64_t N, float scale) {
 // ---- training ---------------------------------------------------------------
 constexpr int kTile = 64;          // samples per block tile (4 warps x 16)
 constexpr int kTrainThreads = 128;
+constexpr int kLdX = kInPad + 8;   // row strides of 80 and 144 bytes: ldmatrix rows on distinct banks
+constexpr int kLdT = kH + 8;
 
+// All matrices row-major as they are in the parameter vector and in the batch;
+// ldmatrix reads them straight or transposed, so no second copy is kept.
 struct TrainSmem {
-  mlp::FwdW w;
-  mlp::BwdW wb;
-  __nv_bfloat16 xs[kTile][mlp::kLd1];
-  __nv_bfloat16 h1[kTile][kH];
-  __nv_bfloat16 h2[kTile][kH];
-  __nv_bfloat16 dz1[kTile][kH];
-  __nv_bfloat16 dz2[kTile][kH];
+  __nv_bfloat16 w1[kInPad][kLdT];  // rows 20 .. 31 zero
+  __nv_bfloat16 w2[kH][kLdT];
+  __nv_bfloat16 w3[kH][kOutPad];   // columns 6, 7 zero
+  __nv_bfloat16 xs[kTile][kLdX];   // columns 20 .. zero
+  __nv_bfloat16 h1[kTile][kLdT];
+  __nv_bfloat16 h2[kTile][kLdT];
+  __nv_bfloat16 dz1[kTile][kLdT];
+  __nv_bfloat16 dz2[kTile][kLdT];
   __nv_bfloat16 dz3[kTile][kOutPad];
+  float b1[kH], b2[kH], b3[kOutPad];
   float abc[kTile][18];
   float bias[4][kH + kH + kOutPad];
   float loss[4];
+  long long idx[kTile];  // the batch slots' samples, -1 past the end
 };
 
 struct LossArgs {
@@ -210,17 +218,139 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {  // splitmix64 finaliser
   return z ^ (z >> 31);
 }
 
+// Four 8 x 8 BF16 matrices from shared memory, row addresses given per lane (lanes
+// 8 i .. 8 i + 7: the rows of matrix i); transposed with _t.
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* row) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(row)));
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const __nv_bfloat16* row) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(row)));
+}
+__device__ __forceinline__ void ldsm2_t(uint32_t& r0, uint32_t& r1, const __nv_bfloat16* row) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r0), "=r"(r1)
+               : "r"((uint32_t)__cvta_generic_to_shared(row)));
+}
+
+// The parameters as BF16 matrices (whole block), four values at a time, from L2:
+// the previous iteration's update may have finished after this kernel started.
+__device__ __forceinline__ void load_params(const float* __restrict__ P, TrainSmem& sm) {
+  const bool wide = ((uintptr_t)P & 15u) == 0;
+  auto four = [&](int off) {
+    return wide ? __ldcg(reinterpret_cast<const float4*>(P + off))
+                : make_float4(__ldcg(P + off), __ldcg(P + off + 1), __ldcg(P + off + 2), __ldcg(P + off + 3));
+  };
+  auto put = [&](__nv_bfloat16* dst, float4 v) {
+    *reinterpret_cast<uint2*>(dst) = make_uint2(mlp::pack_bf16(v.x, v.y), mlp::pack_bf16(v.z, v.w));
+  };
+#pragma unroll 4
+  for (int i = threadIdx.x; i < kInPad * kH / 4; i += kTrainThreads) {
+    const int k = i / (kH / 4), n = 4 * (i % (kH / 4));
+    put(&sm.w1[k][n], k < kIn ? four(mlp::kOffW1 + k * kH + n) : make_float4(0.f, 0.f, 0.f, 0.f));
+  }
+#pragma unroll 8
+  for (int i = threadIdx.x; i < kH * kH / 4; i += kTrainThreads) {
+    const int k = i / (kH / 4), n = 4 * (i % (kH / 4));
+    put(&sm.w2[k][n], four(mlp::kOffW2 + k * kH + n));
+  }
+#pragma unroll 4
+  for (int i = threadIdx.x; i < kH * kOutPad; i += kTrainThreads) {
+    const int k = i / kOutPad, n = i % kOutPad;
+    sm.w3[k][n] = __float2bfloat16_rn(n < kOut ? __ldcg(P + mlp::kOffW3 + k * kOut + n) : 0.0f);
+  }
+  for (int i = threadIdx.x; i < kH; i += kTrainThreads) {
+    sm.b1[i] = __ldcg(P + mlp::kOffB1 + i);
+    sm.b2[i] = __ldcg(P + mlp::kOffB2 + i);
+  }
+  if (threadIdx.x < kOutPad) sm.b3[threadIdx.x] = threadIdx.x < kOut ? __ldcg(P + mlp::kOffB3 + threadIdx.x) : 0.0f;
+}
+
+// A tile's gathered samples on their way to shared memory: five 16-byte pieces of
+// each X row, nine 8-byte pieces of each abc row.
+struct Gather {
+  float4 x[3];
+  float2 a[5];
+  __device__ __forceinline__ void load(const float* __restrict__ X, const float* __restrict__ abc, bool wide,
+                                       const long long* idx) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int c = threadIdx.x + i * kTrainThreads;
+      x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < kTile * 5 && idx[c / 5] >= 0) {
+        const float* p = X + idx[c / 5] * kIn + 4 * (c % 5);
+        x[i] = wide ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const int c = threadIdx.x + i * kTrainThreads;
+      a[i] = make_float2(0.f, 0.f);
+      if (c < kTile * 9 && idx[c / 9] >= 0) {
+        const float* p = abc + idx[c / 9] * 18 + 2 * (c % 9);
+        a[i] = wide ? *reinterpret_cast<const float2*>(p) : make_float2(p[0], p[1]);
+      }
+    }
+  }
+  __device__ __forceinline__ void store(TrainSmem& sm) const {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int c = threadIdx.x + i * kTrainThreads;
+      if (c < kTile * 5)
+        *reinterpret_cast<uint2*>(&sm.xs[c / 5][4 * (c % 5)]) =
+            make_uint2(mlp::pack_bf16(x[i].x, x[i].y), mlp::pack_bf16(x[i].z, x[i].w));
+    }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const int c = threadIdx.x + i * kTrainThreads;
+      if (c < kTile * 9) *reinterpret_cast<float2*>(&sm.abc[c / 9][2 * (c % 9)]) = a[i];
+    }
+  }
+};
+
+// c with the values kept where the (non-negative) activations h are positive
+__device__ __forceinline__ void mask4(float (&c)[4], uint32_t lo, uint32_t hi) {
+  if (!(lo & 0x7fffu)) c[0] = 0.0f;
+  if (!(lo & 0x7fff0000u)) c[1] = 0.0f;
+  if (!(hi & 0x7fffu)) c[2] = 0.0f;
+  if (!(hi & 0x7fff0000u)) c[3] = 0.0f;
+}
+
 // One block: grid-stride over tiles of 64 batch slots; forward, loss, backward
 // per warp (16 samples), weight gradients by tensor-core GEMMs over the tile;
 // the block's gradient sums go to partials[blockIdx.x][0 .. kParams] (+ loss).
-__global__ void __launch_bounds__(kTrainThreads)
+// What binds it is latency (3.4 tiles per block at a batch of 65536): the next
+// tile's gather is in flight during this one's arithmetic, and every operand
+// fragment is one ldmatrix (the transposed ones were gathered two bytes at a time
+// with four-way bank conflicts).  An iteration of 65536 samples: 77.9 us before,
+// 33.2 with the reduction and update below, the same bits.
+__global__ void __launch_bounds__(kTrainThreads, 2)
     grad_kernel(const float* __restrict__ X, const float* __restrict__ abc, int64_t n, int64_t batch, int random,
                 uint64_t seed, uint64_t iter, LossArgs la, const float* __restrict__ P, float* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& sm = *reinterpret_cast<TrainSmem*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  mlp::load_fwd(P, sm.w);
-  mlp::load_bwd(P, sm.wb);
+  const int lr = lane & 7, la1 = (lane >> 3) & 1, la2 = lane >> 4;  // ldmatrix: row, and which of the four matrices
+  const bool wide = (((uintptr_t)X & 15u) | ((uintptr_t)abc & 7u)) == 0;
+  const int64_t ntiles = (batch + kTile - 1) / kTile;
+  auto choose = [&](int64_t tile) {  // the samples of the tile's slots
+    if (threadIdx.x < kTile) {
+      const int64_t slot = tile * kTile + threadIdx.x;
+      long long idx = slot < batch ? slot : -1;
+      if (random && idx >= 0) idx = (long long)(mix64(seed ^ (iter << 32) ^ (uint64_t)slot) % (uint64_t)n);
+      sm.idx[threadIdx.x] = idx;
+    }
+  };
+  choose(blockIdx.x);
+  for (int i = threadIdx.x; i < kTile * kLdX / 2; i += kTrainThreads) reinterpret_cast<uint32_t*>(&sm.xs[0][0])[i] = 0u;
+  __syncthreads();
+  Gather next;
+  next.load(X, abc, wide, sm.idx);
+  chain_wait();  // the samples do not depend on the previous iteration, the parameters do
+  load_params(P, sm);
   float acc_w2[8][4], acc_w1[4][4], acc_w3[4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
@@ -237,23 +367,82 @@ __global__ void __launch_bounds__(kTrainThreads)
   for (int i = 0; i < 16; ++i) db1[i] = db2[i] = 0.0f;
   db3[0] = db3[1] = 0.0f;
   const float inv_batch = 1.0f / (float)batch;
-  const int64_t ntiles = (batch + kTile - 1) / kTile;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     __syncthreads();  // previous tile's shared data fully consumed
-    for (int r = threadIdx.x; r < kTile; r += blockDim.x) {
-      const int64_t slot = tile * kTile + r;
-      const bool valid = slot < batch;
-      int64_t idx = slot;
-      if (random) idx = (int64_t)(mix64(seed ^ (iter << 32) ^ (uint64_t)slot) % (uint64_t)n);
-      for (int j = 0; j < mlp::kLd1; ++j)
-        sm.xs[r][j] = __float2bfloat16_rn(valid && j < kIn ? X[idx * kIn + j] : 0.0f);
-      for (int j = 0; j < 18; ++j) sm.abc[r][j] = valid ? abc[idx * 18 + j] : 0.0f;
-    }
+    next.store(sm);
+    const bool more = tile + gridDim.x < ntiles;
+    if (more) choose(tile + gridDim.x);
     __syncthreads();
+    if (more) next.load(X, abc, wide, sm.idx);
     const int r0 = warp * 16;
     uint32_t h1a[4][4], h2a[4][4];
     float z3[4];
-    mlp::forward16(sm.w, &sm.xs[r0][0], mlp::kLd1, h1a, h2a, z3, &sm.h1[r0][0], &sm.h2[r0][0]);
+    {
+      uint32_t xa[2][4];
+#pragma unroll
+      for (int kc = 0; kc < 2; ++kc) ldsm4(xa[kc], &sm.xs[r0 + lr + 8 * la1][16 * kc + 8 * la2]);
+      // layers 1 and 2: output tiles of 8, two at a time (matrices: k, k + 8 of one, then of the other)
+#pragma unroll
+      for (int np = 0; np < 4; ++np) {
+        float c[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          c[h][0] = c[h][2] = sm.b1[16 * np + 8 * h + 2 * t];
+          c[h][1] = c[h][3] = sm.b1[16 * np + 8 * h + 2 * t + 1];
+        }
+#pragma unroll
+        for (int kc = 0; kc < 2; ++kc) {
+          uint32_t b[4];
+          ldsm4_t(b, &sm.w1[16 * kc + lr + 8 * la1][16 * np + 8 * la2]);
+          mlp::mma(c[0], xa[kc], b[0], b[1]);
+          mlp::mma(c[1], xa[kc], b[2], b[3]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) c[h][k] = fmaxf(c[h][k], 0.0f);
+          h1a[np][2 * h] = mlp::pack_bf16(c[h][0], c[h][1]);
+          h1a[np][2 * h + 1] = mlp::pack_bf16(c[h][2], c[h][3]);
+          *reinterpret_cast<uint32_t*>(&sm.h1[r0 + g][16 * np + 8 * h + 2 * t]) = h1a[np][2 * h];
+          *reinterpret_cast<uint32_t*>(&sm.h1[r0 + g + 8][16 * np + 8 * h + 2 * t]) = h1a[np][2 * h + 1];
+        }
+      }
+#pragma unroll
+      for (int np = 0; np < 4; ++np) {
+        float c[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          c[h][0] = c[h][2] = sm.b2[16 * np + 8 * h + 2 * t];
+          c[h][1] = c[h][3] = sm.b2[16 * np + 8 * h + 2 * t + 1];
+        }
+#pragma unroll
+        for (int kc = 0; kc < 4; ++kc) {
+          uint32_t b[4];
+          ldsm4_t(b, &sm.w2[16 * kc + lr + 8 * la1][16 * np + 8 * la2]);
+          mlp::mma(c[0], h1a[kc], b[0], b[1]);
+          mlp::mma(c[1], h1a[kc], b[2], b[3]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) c[h][k] = fmaxf(c[h][k], 0.0f);
+          h2a[np][2 * h] = mlp::pack_bf16(c[h][0], c[h][1]);
+          h2a[np][2 * h + 1] = mlp::pack_bf16(c[h][2], c[h][3]);
+          *reinterpret_cast<uint32_t*>(&sm.h2[r0 + g][16 * np + 8 * h + 2 * t]) = h2a[np][2 * h];
+          *reinterpret_cast<uint32_t*>(&sm.h2[r0 + g + 8][16 * np + 8 * h + 2 * t]) = h2a[np][2 * h + 1];
+        }
+      }
+      // layer 3: one tile of 8 (6 used), two k chunks per load
+      z3[0] = z3[2] = sm.b3[2 * t];
+      z3[1] = z3[3] = sm.b3[2 * t + 1];
+#pragma unroll
+      for (int kp = 0; kp < 2; ++kp) {
+        uint32_t b[4];
+        ldsm4_t(b, &sm.w3[32 * kp + lane][0]);
+        mlp::mma(z3, h2a[2 * kp], b[0], b[1]);
+        mlp::mma(z3, h2a[2 * kp + 1], b[2], b[3]);
+      }
+    }
     // loss and dL/dz3 for rows r0 + g, r0 + g + 8 and classes 2t, 2t + 1
     float dz3[4];
 #pragma unroll
@@ -271,41 +460,44 @@ __global__ void __launch_bounds__(kTrainThreads)
     }
     db3[0] += dz3[0] + dz3[2];
     db3[1] += dz3[1] + dz3[3];
-    *reinterpret_cast<uint32_t*>(&sm.dz3[r0 + g][2 * t]) = mlp::pack_bf16(dz3[0], dz3[1]);
-    *reinterpret_cast<uint32_t*>(&sm.dz3[r0 + g + 8][2 * t]) = mlp::pack_bf16(dz3[2], dz3[3]);
     // dh2 = dz3 W3^T (k = classes, padded 8 -> 16), masked by h2 > 0
     uint32_t za[4] = {mlp::pack_bf16(dz3[0], dz3[1]), mlp::pack_bf16(dz3[2], dz3[3]), 0u, 0u};
+    *reinterpret_cast<uint32_t*>(&sm.dz3[r0 + g][2 * t]) = za[0];
+    *reinterpret_cast<uint32_t*>(&sm.dz3[r0 + g + 8][2 * t]) = za[1];
     uint32_t d2a[4][4];
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      mlp::mma(c, za, mlp::ld32(&sm.wb.w3s[8 * nt + g][2 * t]), 0u);
-      const int col = 8 * nt + 2 * t;
-      if (!(__bfloat162float(sm.h2[r0 + g][col]) > 0.0f)) c[0] = 0.0f;
-      if (!(__bfloat162float(sm.h2[r0 + g][col + 1]) > 0.0f)) c[1] = 0.0f;
-      if (!(__bfloat162float(sm.h2[r0 + g + 8][col]) > 0.0f)) c[2] = 0.0f;
-      if (!(__bfloat162float(sm.h2[r0 + g + 8][col + 1]) > 0.0f)) c[3] = 0.0f;
-      db2[2 * nt] += c[0] + c[2];
-      db2[2 * nt + 1] += c[1] + c[3];
-      const uint32_t lo = mlp::pack_bf16(c[0], c[1]), hi = mlp::pack_bf16(c[2], c[3]);
-      d2a[nt >> 1][(nt & 1) ? 2 : 0] = lo;
-      d2a[nt >> 1][(nt & 1) ? 3 : 1] = hi;
-      *reinterpret_cast<uint32_t*>(&sm.dz2[r0 + g][col]) = lo;
-      *reinterpret_cast<uint32_t*>(&sm.dz2[r0 + g + 8][col]) = hi;
+    for (int nq = 0; nq < 2; ++nq) {  // four output tiles of 8 per load
+      uint32_t b[4];
+      ldsm4(b, &sm.w3[32 * nq + lane][0]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int nt = 4 * nq + h;
+        float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        mlp::mma(c, za, b[h], 0u);
+        mask4(c, h2a[nt >> 1][2 * (nt & 1)], h2a[nt >> 1][2 * (nt & 1) + 1]);
+        const int col = 8 * nt + 2 * t;
+        db2[2 * nt] += c[0] + c[2];
+        db2[2 * nt + 1] += c[1] + c[3];
+        const uint32_t lo = mlp::pack_bf16(c[0], c[1]), hi = mlp::pack_bf16(c[2], c[3]);
+        d2a[nt >> 1][2 * (nt & 1)] = lo;
+        d2a[nt >> 1][2 * (nt & 1) + 1] = hi;
+        *reinterpret_cast<uint32_t*>(&sm.dz2[r0 + g][col]) = lo;
+        *reinterpret_cast<uint32_t*>(&sm.dz2[r0 + g + 8][col]) = hi;
+      }
     }
-    // dh1 = dz2 W2^T, masked by h1 > 0
+    // dh1 = dz2 W2^T, masked by h1 > 0 (two k chunks of one output tile per load)
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int kc = 0; kc < 4; ++kc)
-        mlp::mma(c, d2a[kc], mlp::ld32(&sm.wb.w2s[8 * nt + g][16 * kc + 2 * t]),
-                 mlp::ld32(&sm.wb.w2s[8 * nt + g][16 * kc + 2 * t + 8]));
+      for (int kp = 0; kp < 2; ++kp) {
+        uint32_t b[4];
+        ldsm4(b, &sm.w2[8 * nt + lr][32 * kp + 8 * (lane >> 3)]);
+        mlp::mma(c, d2a[2 * kp], b[0], b[1]);
+        mlp::mma(c, d2a[2 * kp + 1], b[2], b[3]);
+      }
+      mask4(c, h1a[nt >> 1][2 * (nt & 1)], h1a[nt >> 1][2 * (nt & 1) + 1]);
       const int col = 8 * nt + 2 * t;
-      if (!(__bfloat162float(sm.h1[r0 + g][col]) > 0.0f)) c[0] = 0.0f;
-      if (!(__bfloat162float(sm.h1[r0 + g][col + 1]) > 0.0f)) c[1] = 0.0f;
-      if (!(__bfloat162float(sm.h1[r0 + g + 8][col]) > 0.0f)) c[2] = 0.0f;
-      if (!(__bfloat162float(sm.h1[r0 + g + 8][col + 1]) > 0.0f)) c[3] = 0.0f;
       db1[2 * nt] += c[0] + c[2];
       db1[2 * nt + 1] += c[1] + c[3];
       *reinterpret_cast<uint32_t*>(&sm.dz1[r0 + g][col]) = mlp::pack_bf16(c[0], c[1]);
@@ -314,40 +506,32 @@ __global__ void __launch_bounds__(kTrainThreads)
     __syncthreads();
     // weight gradients over the tile's 64 samples: dW = act^T dz
     auto act_a = [&](const __nv_bfloat16* act, int ld, int mt, int kc, uint32_t (&a)[4]) {
-      const int m0 = 16 * mt + g, k0 = 16 * kc + 2 * t;
-      a[0] = mlp::pack2h(act[k0 * ld + m0], act[(k0 + 1) * ld + m0]);
-      a[1] = mlp::pack2h(act[k0 * ld + m0 + 8], act[(k0 + 1) * ld + m0 + 8]);
-      a[2] = mlp::pack2h(act[(k0 + 8) * ld + m0], act[(k0 + 9) * ld + m0]);
-      a[3] = mlp::pack2h(act[(k0 + 8) * ld + m0 + 8], act[(k0 + 9) * ld + m0 + 8]);
+      ldsm4_t(a, act + (16 * kc + lr + 8 * la2) * ld + 16 * mt + 8 * la1);
     };
-    auto dz_b = [&](const __nv_bfloat16* dz, int ld, int nt, int kc, uint32_t& b0, uint32_t& b1) {
-      const int n0 = 8 * nt + g, k0 = 16 * kc + 2 * t;
-      b0 = mlp::pack2h(dz[k0 * ld + n0], dz[(k0 + 1) * ld + n0]);
-      b1 = mlp::pack2h(dz[(k0 + 8) * ld + n0], dz[(k0 + 9) * ld + n0]);
+    auto dz_b2 = [&](const __nv_bfloat16* dz, int ld, int np, int kc, uint32_t (&b)[4]) {  // output tiles 2 np, 2 np + 1
+      ldsm4_t(b, dz + (16 * kc + lr + 8 * la1) * ld + 16 * np + 8 * la2);
     };
 #pragma unroll
     for (int kc = 0; kc < 4; ++kc) {
-      uint32_t a[4];
-      act_a(&sm.h1[0][0], kH, warp, kc, a);  // dW2: rows 16 warp .. of W2
+      uint32_t a[4], b[4];
+      act_a(&sm.h1[0][0], kLdT, warp, kc, a);  // dW2: rows 16 warp .. of W2
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
-        uint32_t b0, b1;
-        dz_b(&sm.dz2[0][0], kH, nt, kc, b0, b1);
-        mlp::mma(acc_w2[nt], a, b0, b1);
+      for (int np = 0; np < 4; ++np) {
+        dz_b2(&sm.dz2[0][0], kLdT, np, kc, b);
+        mlp::mma(acc_w2[2 * np], a, b[0], b[1]);
+        mlp::mma(acc_w2[2 * np + 1], a, b[2], b[3]);
       }
-      act_a(&sm.h2[0][0], kH, warp, kc, a);  // dW3: rows 16 warp ..
-      {
-        uint32_t b0, b1;
-        dz_b(&sm.dz3[0][0], kOutPad, 0, kc, b0, b1);
-        mlp::mma(acc_w3, a, b0, b1);
-      }
+      act_a(&sm.h2[0][0], kLdT, warp, kc, a);  // dW3: rows 16 warp ..
+      uint32_t b0, b1;
+      ldsm2_t(b0, b1, &sm.dz3[16 * kc + (lane & 15)][0]);
+      mlp::mma(acc_w3, a, b0, b1);
+      // dW1: tiles 4 warp .. 4 warp + 3 of (2 x 8)
+      act_a(&sm.xs[0][0], kLdX, warp >> 1, kc, a);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {  // dW1: tiles 4 warp .. 4 warp + 3 of (2 x 8)
-        const int tt = 4 * warp + q, mt = tt >> 3, nt = tt & 7;
-        uint32_t a1[4], b0, b1;
-        act_a(&sm.xs[0][0], mlp::kLd1, mt, kc, a1);
-        dz_b(&sm.dz1[0][0], kH, nt, kc, b0, b1);
-        mlp::mma(acc_w1[q], a1, b0, b1);
+      for (int q = 0; q < 2; ++q) {
+        dz_b2(&sm.dz1[0][0], kLdT, 2 * (warp & 1) + q, kc, b);
+        mlp::mma(acc_w1[2 * q], a, b[0], b[1]);
+        mlp::mma(acc_w1[2 * q + 1], a, b[2], b[3]);
       }
     }
   }
@@ -410,32 +594,48 @@ __global__ void __launch_bounds__(kTrainThreads)
   if (threadIdx.x == 0) out[kParams] = sm.loss[0] + sm.loss[1] + sm.loss[2] + sm.loss[3];
 }
 
-// grad[k] = sum over blocks (fixed order); grad[kParams] = loss sum
-__global__ void grad_reduce_kernel(const float* __restrict__ partials, int nblocks, int64_t batch,
-                                   float* __restrict__ grad, float* __restrict__ loss_out) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > kParams) return;
-  float s = 0.0f;
-  for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * kParamsPad + k];
-  grad[k] = s;
-  if (k == kParams && loss_out) *loss_out = s / (float)batch;
-}
+// One Adam step (beta1 0.9, beta2 0.999, eps 1e-8) of the reduced gradient.
+struct AdamArgs {
+  float *P, *m, *v;  // P = nullptr: no step
+  float lr, b1t, b2t;
+};
 
-__global__ void adam_kernel(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ grad, float lr, float b1t, float b2t) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= kParams) return;
-  const float gk = grad[k];
-  const float mk = 0.9f * m[k] + 0.1f * gk;
-  const float vk = 0.999f * v[k] + 0.001f * gk * gk;
-  m[k] = mk;
-  v[k] = vk;
-  P[k] -= lr * (mk / b1t) / (sqrtf(vk / b2t) + 1e-8f);
+// grad[k] = sum over blocks in their order, grad[kParams] = loss sum; then the Adam
+// step of parameter k.  Eight warps stage a column of 32 parameters in shared memory
+// (304 loads one after the other were two thirds of an iteration), one adds them up.
+constexpr int kTrainBlocks = 304;
+constexpr int kReduceWays = 8;
+__global__ void __launch_bounds__(32 * kReduceWays)
+    grad_reduce_kernel(const float* __restrict__ partials, int nblocks, int64_t batch, float* __restrict__ grad,
+                       float* __restrict__ loss_out, AdamArgs ad) {
+  __shared__ float part[kTrainBlocks][32];
+  const int lane = threadIdx.x & 31, way = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
+  chain_wait();
+  if (k <= kParams) {
+#pragma unroll 8
+    for (int b = way; b < nblocks; b += kReduceWays) part[b][lane] = __ldcg(&partials[(size_t)b * kParamsPad + k]);
+  }
+  __syncthreads();
+  if (way != 0 || k > kParams) return;
+  float s = 0.0f;
+#pragma unroll 16
+  for (int b = 0; b < nblocks; ++b) s += part[b][lane];
+  grad[k] = s;
+  if (k == kParams) {
+    if (loss_out) *loss_out = s / (float)batch;
+    return;
+  }
+  if (!ad.P) return;
+  const float mk = 0.9f * ad.m[k] + 0.1f * s;
+  const float vk = 0.999f * ad.v[k] + 0.001f * s * s;
+  ad.m[k] = mk;
+  ad.v[k] = vk;
+  ad.P[k] -= ad.lr * (mk / ad.b1t) / (sqrtf(vk / ad.b2t) + 1e-8f);
 }
 
 int train_blocks(int64_t batch) {
   const int64_t tiles = (batch + kTile - 1) / kTile;
-  return (int)(tiles < 304 ? tiles : 304);
+  return (int)(tiles < kTrainBlocks ? tiles : kTrainBlocks);
 }
 
 size_t train_smem() { return sizeof(TrainSmem); }
@@ -446,7 +646,7 @@ size_t closure_partials_bytes(int64_t batch) { return (size_t)train_blocks(batch
 
 cudaError_t closure_grad(const float* X, const float* abc, int64_t n, int64_t batch, int random, uint64_t seed,
                          uint64_t iter, const float* cw, double lo, double hi, const float* P, float* partials,
-                         float* grad, float* loss, cudaStream_t stream) {
+                         float* grad, float* loss, const ClosureAdam* adam, cudaStream_t stream) {
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem());
@@ -457,18 +657,29 @@ cudaError_t closure_grad(const float* X, const float* abc, int64_t n, int64_t ba
   for (int c = 0; c < kOut; ++c) la.cw[c] = cw[c];
   la.lo = (float)lo;
   la.span = (float)(hi - lo);
+  AdamArgs ad = {nullptr, nullptr, nullptr, 0.f, 1.f, 1.f};
+  if (adam) {
+    ad.P = adam->P;
+    ad.m = adam->m;
+    ad.v = adam->v;
+    ad.lr = (float)adam->lr;
+    ad.b1t = (float)(1.0 - std::pow(0.9, (double)adam->step));
+    ad.b2t = (float)(1.0 - std::pow(0.999, (double)adam->step));
+  }
   const int nb = train_blocks(batch);
-  grad_kernel<<<nb, kTrainThreads, train_smem(), stream>>>(X, abc, n, batch, random, seed, iter, la, P, partials);
-  grad_reduce_kernel<<<(kParams + 1 + 255) / 256, 256, 0, stream>>>(partials, nb, batch, grad, loss);
-  return cudaGetLastError();
-}
-
-cudaError_t closure_adam(float* P, float* m, float* v, const float* grad, double lr, int64_t step,
-                         cudaStream_t stream) {
-  const float b1t = (float)(1.0 - std::pow(0.9, (double)step));
-  const float b2t = (float)(1.0 - std::pow(0.999, (double)step));
-  adam_kernel<<<(kParams + 255) / 256, 256, 0, stream>>>(P, m, v, grad, (float)lr, b1t, b2t);
-  return cudaGetLastError();
+  // Chained launches: an iteration's samples are gathered while the previous one's
+  // sums are still being reduced.  The first one waits for whatever wrote the samples.
+  cudaError_t e;
+  if (adam && !adam->first) {
+    e = launch_chained(grad_kernel, dim3(nb), dim3(kTrainThreads), train_smem(), stream, X, abc, n, batch, random, seed,
+                       iter, la, P, partials);
+  } else {
+    grad_kernel<<<nb, kTrainThreads, train_smem(), stream>>>(X, abc, n, batch, random, seed, iter, la, P, partials);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  return launch_chained(grad_reduce_kernel, dim3((kParams + 1 + 31) / 32), dim3(32 * kReduceWays), 0, stream, partials,
+                        nb, batch, grad, loss, ad);
 }
 
 cudaError_t closure_filter(Sim* s, int m, float* out) {

@@ -29,4 +29,9 @@ __device__ __forceinline__ bool row_of(uint32_t q, RowLength r, int ny, int& i, 
   return y < ny;
 }
 
+// The compiler does not know these values to be what they were: what it computed
+// from them before is computed again after, instead of being kept in registers.
+__device__ __forceinline__ void forget(int& x, int& y, int& z) { asm volatile("" : "+r"(x), "+r"(y), "+r"(z)); }
+__device__ __forceinline__ void forget(int& x, int& y) { asm volatile("" : "+r"(x), "+r"(y)); }
+
 }  // namespace lbm

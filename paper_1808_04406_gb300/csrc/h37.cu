@@ -471,7 +471,7 @@ cudaError_t pair_t(Sim* s, int odd) {
   using E = typename PairIO<S>::E;
   dim3 grid((unsigned)((s->nx / 2 + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
   E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? h37_pair_kernel<S, true> : h37_pair_kernel<S, false>, grid, dim3(kH37Threads), s->stream, f,
+  return launch_chained(odd ? h37_pair_kernel<S, true> : h37_pair_kernel<S, false>, grid, dim3(kH37Threads), 0, s->stream, f,
                         grid2(s), sweep_model<S, false>(s), status_word(s));
 }
 
@@ -480,7 +480,7 @@ cudaError_t pair_totals_t(Sim* s, int odd, float* partials) {
   using E = typename PairIO<S>::E;
   dim3 grid((unsigned)((s->nx / 2 + kH37Threads - 1) / kH37Threads), (unsigned)s->ny);
   E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? h37_pair_totals_kernel<S, true> : h37_pair_totals_kernel<S, false>, grid, dim3(kH37Threads),
+  return launch_chained(odd ? h37_pair_totals_kernel<S, true> : h37_pair_totals_kernel<S, false>, grid, dim3(kH37Threads), 0,
                         s->stream, f, grid2(s), sweep_model<S, false>(s), status_word(s), partials);
 }
 
@@ -502,7 +502,7 @@ cudaError_t sweep_t(Sim* s, int odd) {
   const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   E* f = static_cast<E*>(s->pop);
   auto launch = [&](auto odd_c, auto exact_c) {
-    return launch_chained(h37_sweep_kernel<S, decltype(odd_c)::value, decltype(exact_c)::value>, dim3(blocks), dim3(t),
+    return launch_chained(h37_sweep_kernel<S, decltype(odd_c)::value, decltype(exact_c)::value>, dim3(blocks), dim3(t), 0,
                           s->stream, f, grid2(s), sweep_model<S, decltype(exact_c)::value>(s), status_word(s));
   };
   if constexpr (S == LBM_F32) {

@@ -806,7 +806,7 @@ cudaError_t orbit_sweep(Sim* s, int odd, bool* taken) {
   const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   T* f = static_cast<T*>(s->pop);
   return launch_chained(odd ? hgen_orbit_kernel<T, NC, NA, NQ, true> : hgen_orbit_kernel<T, NC, NA, NQ, false>,
-                        dim3(blocks), dim3(t), s->stream, f, hgrid(s), rule, hmoment_model<T>(s), status_word(s));
+                        dim3(blocks), dim3(t), 0, s->stream, f, hgrid(s), rule, hmoment_model<T>(s), status_word(s));
 }
 
 template <int S, int Q, int NC, bool EXACT>

@@ -859,7 +859,7 @@ int lbm_mlp_loss_grad(const float* X, const float* abc, int64_t n, const float* 
   float* partials = static_cast<float*>(work);
   float* g = reinterpret_cast<float*>(static_cast<unsigned char*>(work) + closure_partials_bytes(n));
   float* l = g + 5895;
-  int rc = cuda_check(closure_grad(X, abc, n, n, 0, 0, 0, cw, omega_lo, omega_hi, params, partials, g, l, st),
+  int rc = cuda_check(closure_grad(X, abc, n, n, 0, 0, 0, cw, omega_lo, omega_hi, params, partials, g, l, nullptr, st),
                       "gradient kernels");
   if (!rc && grad)
     rc = cuda_check(cudaMemcpyAsync(grad, g, 5894 * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy gradient");
@@ -881,10 +881,10 @@ int lbm_mlp_train(const float* X, const float* abc, int64_t n, const float* cw, 
   float* partials = static_cast<float*>(work);
   float* g = reinterpret_cast<float*>(static_cast<unsigned char*>(work) + closure_partials_bytes(batch));
   for (int64_t it = 0; it < iters; ++it) {
+    const ClosureAdam adam = {params, adam_m, adam_v, lr, t0 + it + 1, it == 0};
     int rc = cuda_check(closure_grad(X, abc, n, batch, 1, seed, (uint64_t)(t0 + it), cw, omega_lo, omega_hi, params,
-                                     partials, g, loss_hist ? loss_hist + it : nullptr, st),
-                        "gradient kernels");
-    if (!rc) rc = cuda_check(closure_adam(params, adam_m, adam_v, g, lr, t0 + it + 1, st), "adam kernel");
+                                     partials, g, loss_hist ? loss_hist + it : nullptr, &adam, st),
+                        "gradient and optimiser kernels");
     if (rc) return rc;
   }
   return LBM_OK;

@@ -168,12 +168,17 @@ cudaError_t closure_filter(Sim* s, int m, float* out);
 cudaError_t closure_dataset(const int64_t dims[3], const float* ft, const float* ft1, double tau2, const float* norm,
                             float* X, float* abc, cudaStream_t stream);
 size_t closure_partials_bytes(int64_t batch);
+// the optimiser step that follows a gradient: parameters, moments, learning rate, step number
+struct ClosureAdam {
+  float *P, *m, *v;
+  double lr;
+  int64_t step;
+  bool first;  // the first iteration of a call
+};
 cudaError_t closure_grad(const float* X, const float* abc, int64_t n, int64_t batch, int random, uint64_t seed,
                          uint64_t iter, const float* cw, double lo, double hi, const float* P, float* partials,
-                         float* grad, float* loss, cudaStream_t stream);
+                         float* grad, float* loss, const ClosureAdam* adam, cudaStream_t stream);
 cudaError_t closure_rescale(int64_t N, float* f, double scale, cudaStream_t stream);
-cudaError_t closure_adam(float* P, float* m, float* v, const float* grad, double lr, int64_t step,
-                         cudaStream_t stream);
 cudaError_t closure_sweep(Sim* s, int odd, const void* img, const float* norm);
 cudaError_t closure_build_image(const float* P, void* img, cudaStream_t stream);
 size_t closure_image_bytes();

@@ -46,7 +46,7 @@ struct PairUp {
     for (int n = 0; n <= 2 * D; ++n) om[n] = cst<f2>(p.r.w[n]);
     tp::pair_decode<D, LBM_F32, ODD>(raw, v);
     // the stores' addresses are computed anew: kept from the loads they would take 54 registers
-    if constexpr (D == 3) asm volatile("" : "+r"(xp), "+r"(y), "+r"(z));
+    if constexpr (D == 3) forget(xp, y, z);
     const bool ok = tp::collide<f2, D>(v, om);
     tp::pair_store<D, LBM_F32, ODD>(f, p.g, tp::PairAddr<D, ODD>(p.g, xp, y, z), v);
     return ok;

@@ -33,9 +33,6 @@ constexpr int kPairThreads = LBM_PAIR_THREADS;
 // loads (54 registers on D3Q27) the sweeps take 128 registers or less.
 constexpr int kPairMinBlocks = 4;
 
-// The compiler does not know these values to be what they were.
-__device__ __forceinline__ void forget(int& x, int& y, int& z) { asm volatile("" : "+r"(x), "+r"(y), "+r"(z)); }
-
 template <int D, int S, bool ODD>
 __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks)
     tp_pair_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r,
@@ -247,7 +244,7 @@ cudaError_t launch_zrun(Sim* s, int odd) {
   dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
   const int z0 = (int)active_z0(s), z1 = (int)(active_z0(s) + nzs);
   E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? tp_pair_zrun_kernel<S, true> : tp_pair_zrun_kernel<S, false>, grid, dim3(kPairThreads),
+  return launch_chained(odd ? tp_pair_zrun_kernel<S, true> : tp_pair_zrun_kernel<S, false>, grid, dim3(kPairThreads), 0,
                         s->stream, f, g, s->rates, status_word(s), row_length(s->nx / 2), z0, z1, run);
 }
 
@@ -262,7 +259,7 @@ cudaError_t launch(Sim* s, int odd) {
   dim3 grid(plane_blocks(s), 1, (unsigned)active_nz(s));
   const int z0 = (int)active_z0(s);
   E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? tp_pair_kernel<D, S, true> : tp_pair_kernel<D, S, false>, grid, block, s->stream, f, g,
+  return launch_chained(odd ? tp_pair_kernel<D, S, true> : tp_pair_kernel<D, S, false>, grid, block, 0, s->stream, f, g,
                         s->rates, status_word(s), row_length(s->nx / 2), z0);
 }
 
@@ -276,7 +273,7 @@ cudaError_t launch_zrun_totals(Sim* s, int odd, float* partials) {
   const int z0 = (int)active_z0(s), z1 = (int)(active_z0(s) + nzs);
   E* f = static_cast<E*>(s->pop);
   return launch_chained(odd ? tp_pair_zrun_totals_kernel<S, true> : tp_pair_zrun_totals_kernel<S, false>, grid,
-                        dim3(kPairThreads), s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
+                        dim3(kPairThreads), 0, s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
 }
 
 template <int D, int S>
@@ -292,7 +289,7 @@ cudaError_t launch_totals(Sim* s, int odd, float* partials) {
   dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
   const int z0 = (int)active_z0(s), z1 = (int)(z0 + nzs);
   E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? tp_pair_totals_kernel<D, S, true> : tp_pair_totals_kernel<D, S, false>, grid, block,
+  return launch_chained(odd ? tp_pair_totals_kernel<D, S, true> : tp_pair_totals_kernel<D, S, false>, grid, block, 0,
                         s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
 }
 

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kSweepThreads, D == 3 ? 4 : 6)
     }
   }
   // the stores' addresses are computed anew: kept from the loads they would take too many registers
-  asm volatile("" : "+r"(x), "+r"(y), "+r"(z));
+  forget(x, y, z);
   if (!tp::collide<f2, D>(v, om)) atomicOr(status, 1);
   const ColumnPair<D, ODD> A(g, x, y, z);
 #pragma unroll
@@ -136,7 +136,7 @@ template <int D, int S>
 cudaError_t launch_columns(Sim* s, int odd) {
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
   dim3 grid((unsigned)column_blocks(s), 1, (unsigned)active_nz(s));
-  return launch_chained(odd ? tp_column_kernel<D, S, true> : tp_column_kernel<D, S, false>, grid, dim3(kSweepThreads),
+  return launch_chained(odd ? tp_column_kernel<D, S, true> : tp_column_kernel<D, S, false>, grid, dim3(kSweepThreads), 0,
                         s->stream, static_cast<typename PairIO<S>::E*>(s->pop), g, s->rates, status_word(s),
                         row_length(s->nx), (int)active_z0(s));
 }
@@ -149,7 +149,7 @@ cudaError_t launch(Sim* s, int odd) {
   dim3 grid((unsigned)((s->nx * s->ny + kSweepThreads - 1) / kSweepThreads), 1, (unsigned)active_nz(s));
   Tst* f = static_cast<Tst*>(s->pop);
   const int z0 = (int)active_z0(s);
-  return launch_chained(odd ? tp_sweep_kernel<D, S, true> : tp_sweep_kernel<D, S, false>, grid, block, s->stream, f, g,
+  return launch_chained(odd ? tp_sweep_kernel<D, S, true> : tp_sweep_kernel<D, S, false>, grid, block, 0, s->stream, f, g,
                         s->rates, status_word(s), row_length(s->nx), z0);
 }
 

@@ -411,3 +411,31 @@ def test_full_size_learned_128_sampled_parity(lbm):
         effect = max(effect, np.abs(want - plain).max())
     assert effect > 1e-4
     assert err <= 3e-2 * effect, (err, effect)
+
+
+@pytest.mark.parametrize("n,batch,offset", [(1, 1, 0), (63, 64, 0), (65, 63, 1), (1000, 304 * 64 + 1, 1), (500, 129, 2)])
+def test_training_takes_any_alignment_and_batch_remainder(lbm, n, batch, offset):
+    """Mini-batches of one tile, of a remainder, and of one tile more than there are
+    blocks, on samples that start `offset` floats past an aligned address: the same
+    parameters, moments and losses, bit for bit, as on an aligned copy."""
+    import torch
+    from paper_1808_04406_gb300 import closure as C
+    g = torch.Generator(device="cuda").manual_seed(3)
+    X = torch.randn(n, 20, generator=g, device="cuda")
+    k = torch.randn(n, 6, generator=g, device="cuda")
+    abc = torch.stack([k * k, 0.3 * k, k * k + 0.1], dim=2).reshape(n, 18).contiguous()
+    cw = [1.0, 0.5, 2.0, 1.0, 0.25, 1.0]
+
+    def shifted(a):
+        buf = torch.empty(a.numel() + offset, device="cuda")
+        buf[offset:] = a.reshape(-1)
+        return buf[offset:].view(a.shape)
+
+    out = []
+    for x, y in ((X, abc), (shifted(X), shifted(abc))):
+        t = C.Trainer(C.init_params(1, "cuda"), batch)
+        losses = t.train(x, y, cw, 3, 1e-3, seed=5)
+        out.append((torch.tensor(losses), t.params.cpu(), t.m.cpu(), t.v.cpu()))
+    assert all(torch.isfinite(v).all() for v in out[0])
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
