@@ -9,6 +9,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "flat_index.cuh"
 #include "h37_moments.cuh"
 #include "pair_io.cuh"
 #include "pdl.cuh"
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(kH37Threads)
   const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
   chain_wait();
   if (node >= (uint32_t)g.N) return;
-  const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
+  int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
   T v[h37::kQ];
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j)
@@ -160,12 +161,16 @@ __global__ void __launch_bounds__(kH37Threads)
     ok = update_values<T, kScaled>(v, m, static_cast<T*>(nullptr));
   if (!ok) atomicOr(status, 1);
   // even sweep: population i goes to slot (x, opp(i)); odd sweep: to slot (x + e_i, i)
-  h37::SrStream rs(rounding(m).seed, node);
+  // 16-bit storage: the stores' addresses anew, for twice the warps (the correctly
+  // rounded FP32 update is better off with them kept: 128^2 4.0 us a step, 4.6 so)
+  if constexpr (kScaled) forget(x, y);
+  const uint32_t own = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
+  h37::SrStream rs(rounding(m).seed, own);
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j) {
     const T val = ODD ? v[j] : v[h37::opp(j)];
     const auto e = kScaled && rounding(m).sround ? restore_sr<S>(val, rs.next()) : restore<S>(val);
-    f[(size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : node)] = e;
+    f[(size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : own)] = e;
   }
 }
 
@@ -176,8 +181,12 @@ __global__ void __launch_bounds__(kH37Threads)
 // directions with odd e_x (an aligned access; the periodic wrap preserves the
 // parity because nx is even) and takes two 1-element accesses for the 17 with
 // even e_x.
+//
+// 4 blocks per SM: with the stores' addresses computed anew instead of kept from the
+// loads the kernel takes 112 registers (168 before, at 3 blocks: FP16 1024^2 29.5
+// us a step, 27.7 so).
 #ifndef LBM_H37_PAIR_MINB
-#define LBM_H37_PAIR_MINB 3  // 168 registers (a few words spill): 12 warps per SM
+#define LBM_H37_PAIR_MINB 4
 #endif
 // The update of pair xp of row blockIdx.y; with TOT the pair's conserved
 // moments (drho, j_x, j_y, both lanes) go to mom[0..2].
@@ -187,8 +196,8 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
                                                 f2* mom) {
   using IO = PairIO<S>;
   using E = typename IO::E;
-  const int y = blockIdx.y;
-  const int x0 = 2 * xp + (ODD ? 1 : 0);
+  int y = blockIdx.y;
+  int x0 = 2 * xp + (ODD ? 1 : 0);
   const int nx = g.nx;
   auto wrapx = [&](int x) { return x < 0 ? x + nx : (x >= nx ? x - nx : x); };
   auto rowof = [&](int ey) -> uint32_t {
@@ -215,6 +224,7 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
   }
   const bool ok = update_values<f2, IO::kScaled>(v, m, TOT ? mom : nullptr);
   if (!ok) atomicOr(status, 1);
+  forget(x0, y);
   // the pair's own nodes (for the stochastic-rounding bits)
   const uint32_t n0 = (uint32_t)x0 + (uint32_t)nx * (uint32_t)y, n1 = (uint32_t)wrapx(x0 + 1) + (uint32_t)nx * (uint32_t)y;
   h37::SrStream rs0(rounding(m).seed, n0), rs1(rounding(m).seed, n1);
