@@ -21,6 +21,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "flat_index.cuh"
 #include "lbm_internal.cuh"
 #include "mlp.cuh"
 #include "pdl.cuh"
@@ -725,6 +726,10 @@ cudaError_t closure_dataset(const int64_t dims[3], const float* ft, const float*
 namespace {
 
 constexpr int kLearnThreads = 128;
+// Blocks per SM of the tcgen05 sweep: features and activations share one tile (37 KB of
+// shared memory a block) and all layers the same 64 accumulator columns, so that 5 fit
+// at 96 registers.
+constexpr int kTcBlocks = 5;
 
 #ifndef LBM_LEARN_MINB
 #define LBM_LEARN_MINB 4  // 128 registers (a few words spill to L1): 16 warps per SM
@@ -859,17 +864,25 @@ __global__ void __launch_bounds__(kLearnThreads, LBM_LEARN_MINB)
 }
 
 // ---- the same sweep with the network on tcgen05 -----------------------------
-// A 128-node tile is one M = 128 MMA chain: features A1[128 x 32], hidden
-// activations A2 / A3[128 x 80] (shared, K-major core-matrix layout), weights
-// B1[64 x 32], B2[64 x 80], B3[16 x 80].  Biases ride in three extra K columns
+// A 128-node tile is one M = 128 MMA chain: features [128 x 32] and hidden
+// activations [128 x 80], one after the other in the same tile (shared, K-major
+// core-matrix layout, rows of 80), weights B1[64 x 32], B2[64 x 80], B3[16 x 80].  Biases ride in three extra K columns
 // (BF16 high, middle and low parts) against constant-one inputs, so the FP32
 // accumulators hold W x + b with the bias to FP32 precision.
-// Accumulators: tensor-memory columns 0..63 (layers 1 and 2), 64..79 (layer 3).
+// Accumulators: tensor-memory columns 0..63 (layers 1 and 2), 0..15 (layer 3).
+//
+// A tile is a serial chain (loads, moments, three layers, relaxation, stores), so the
+// sweep is bounded by the latencies that the blocks of an SM cannot cover for each
+// other: issue slots 61 % busy, HBM 40 %.  128^3, us a step: 142 at 4 blocks per SM with
+// each tile's loads going to HBM; 139 at 5; 133 with the next tile's lines prefetched
+// into L2; 124 with the tile's coordinates by reciprocals instead of four 64-bit
+// divisions, no barrier after the last layer (each thread has seen it complete) and
+// chained launches.
 namespace tcimg {
 constexpr int kK1 = 32, kK2 = 80, kN3 = 16;
 constexpr int kB1 = 0, kB2 = kB1 + 64 * kK1 * 2, kB3 = kB2 + 64 * kK2 * 2, kBytes = kB3 + kN3 * kK2 * 2;  // 16896
-constexpr int kA1Bytes = 128 * kK1 * 2, kA2Bytes = 128 * kK2 * 2;
-constexpr uint32_t kCols = 128;
+constexpr int kABytes = 128 * kK2 * 2;
+constexpr uint32_t kCols = 64;
 constexpr int kWaitPolls = 1 << 20;
 }  // namespace tcimg
 
@@ -944,8 +957,7 @@ __global__ void build_tc_image_kernel(const float* __restrict__ P, unsigned char
 
 struct TcSmem {
   unsigned char w[tcimg::kBytes];
-  unsigned char a1[tcimg::kA1Bytes];
-  unsigned char a2[tcimg::kA2Bytes];
+  unsigned char a[tcimg::kABytes];  // features, then the activations of each layer
   uint64_t mbar;
   uint32_t tbase;
 };
@@ -955,13 +967,14 @@ __device__ __forceinline__ void put8(unsigned char* tile, int K, int r, int kgro
   *reinterpret_cast<uint4*>(tile + tc05::core_offset(r, 8 * kgroup, K)) = v;
 }
 
-// One thread issues the MMAs of one layer (K / 16 slices) and commits them.
+// One thread issues the MMAs of one layer (K / 16 slices) and commits them.  The
+// activation tile's rows are kK2 long whatever the layer uses of them.
 __device__ __forceinline__ void issue_layer(uint32_t d_tmem, const unsigned char* a, const unsigned char* b, int K,
                                             uint32_t idesc, uint64_t* mbar) {
   const uint32_t a0 = tc05::smem_u32(a), b0 = tc05::smem_u32(b), sbo = (uint32_t)(K / 8) * 128;
   for (int s = 0; s < K / 16; ++s)
-    tc05::mma(d_tmem, tc05::make_desc(a0 + 256 * s, 128, sbo), tc05::make_desc(b0 + 256 * s, 128, sbo), idesc,
-              s > 0 ? 1u : 0u);
+    tc05::mma(d_tmem, tc05::make_desc(a0 + 256 * s, 128, (uint32_t)(tcimg::kK2 / 8) * 128),
+              tc05::make_desc(b0 + 256 * s, 128, sbo), idesc, s > 0 ? 1u : 0u);
   tc05::commit(mbar);
 }
 
@@ -986,25 +999,35 @@ __device__ __forceinline__ void relu_to_tile(uint32_t taddr, unsigned char* a2, 
   }
 }
 
+// Warp w's 32 nodes of the tile: lane j < 27 asks for the line of L2 that holds the first
+// one's population j (the neighbouring warps' lines hold what a shifted slot adds).
 template <bool ODD>
-__global__ void __launch_bounds__(kLearnThreads, 4)
+__device__ __forceinline__ void prefetch_tile(const float* f, const tp::Grid& g, int x, int y, int z, int lane) {
+  if (lane >= 27 || x >= g.nx) return;
+  uint32_t slot;
+  if (ODD) {
+    y += lane / 3 % 3 - 1;
+    z += lane / 9 - 1;
+    y = y < 0 ? g.ny - 1 : (y >= g.ny ? 0 : y);
+    z = z < 0 ? g.nz - 1 : (z >= g.nz ? 0 : z);
+  }
+  slot = (uint32_t)x + (uint32_t)g.nx * ((uint32_t)y + (uint32_t)g.ny * (uint32_t)z);
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(f + (size_t)lane * g.N + slot));
+}
+
+template <bool ODD>
+__global__ void __launch_bounds__(kLearnThreads, kTcBlocks)
     learned_tc_kernel(float* __restrict__ f, tp::Grid g, Rates r, const unsigned char* __restrict__ img,
-                      const float* __restrict__ norm, int* __restrict__ status) {
+                      const float* __restrict__ norm, int* __restrict__ status, RowLength xtiles, RowLength rows) {
   using namespace tcimg;
   extern __shared__ __align__(16) unsigned char tc_smem_raw[];
   // operand tiles start on 128-byte boundaries (descriptors need 16)
   TcSmem& sm = *reinterpret_cast<TcSmem*>(tc_smem_raw + ((128u - (tc05::smem_u32(tc_smem_raw) & 127u)) & 127u));
   const int tid = threadIdx.x, warp = tid >> 5;
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(img);
-    uint4* dst = reinterpret_cast<uint4*>(sm.w);
-    for (int i = tid; i < kBytes / 16; i += blockDim.x) dst[i] = src[i];
-  }
-  // constant K columns of this thread's rows: A1 k 24..31 zero; A2 k 64..66 one, 67..79 zero
+  // constant K columns of this thread's row: k 64..66 one, 67..79 zero
   const uint32_t one2 = mlp::pack_bf16(1.0f, 1.0f), one0 = mlp::pack_bf16(1.0f, 0.0f);
-  put8(sm.a1, kK1, tid, 3, make_uint4(0u, 0u, 0u, 0u));
-  put8(sm.a2, kK2, tid, 8, make_uint4(one2, one0, 0u, 0u));
-  put8(sm.a2, kK2, tid, 9, make_uint4(0u, 0u, 0u, 0u));
+  put8(sm.a, kK2, tid, 8, make_uint4(one2, one0, 0u, 0u));
+  put8(sm.a, kK2, tid, 9, make_uint4(0u, 0u, 0u, 0u));
   if (warp == 0) {
     tc05::alloc(&sm.tbase, kCols);
     tc05::relinquish();
@@ -1013,27 +1036,38 @@ __global__ void __launch_bounds__(kLearnThreads, 4)
     tc05::mbar_init(&sm.mbar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  chain_wait();
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(img);
+    uint4* dst = reinterpret_cast<uint4*>(sm.w);
+    for (int i = tid; i < kBytes / 16; i += blockDim.x) dst[i] = src[i];
+  }
   tc05::fence_before();
   __syncthreads();
   tc05::fence_after();
   const uint32_t tmem = sm.tbase;
   const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);  // this warp's lane quarter
   const uint32_t id64 = tc05::idesc_bf16(128, 64), id16 = tc05::idesc_bf16(128, kN3);
-  const int xtiles = (g.nx + kLearnThreads - 1) / kLearnThreads;
-  const int64_t ntile = (int64_t)xtiles * g.ny * g.nz;
+  const uint32_t ntile = xtiles.n * (uint32_t)g.ny * (uint32_t)g.nz;
+  auto tile_at = [&](uint32_t tile, int& xt, int& y, int& z) {
+    uint32_t rest;
+    const uint32_t yz = divide(tile, xtiles, rest);
+    xt = (int)rest;
+    z = (int)divide(yz, rows, rest);
+    y = (int)rest;
+  };
   const float tau2m = 1.0f / (float)r.w[2] - 0.5f;
   const float x_tau = (tau2m - norm[kIn - 1]) * norm[2 * kIn - 1];  // the one standardised feature
   const float lo = norm[2 * kIn], span = norm[2 * kIn + 1] - norm[2 * kIn];
   const float om2 = (float)r.w[2];
   uint32_t phase = 0;
   int bad = 0;
-  for (int64_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-    const int xt = (int)(tile % xtiles);
-    const int64_t yz = tile / xtiles;
-    const int y = (int)(yz % g.ny), z = (int)(yz / g.ny);
+  for (uint32_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    int xt, y, z;
+    tile_at(tile, xt, y, z);
     const int x = xt * kLearnThreads + tid;
     const bool active = x < g.nx;
-    const int xc = active ? x : 0;
+    int xc = active ? x : 0;
     float v[27];
     if (active) {
       // the slots of this node in the parity's AA layout: per-axis wrapped
@@ -1044,10 +1078,15 @@ __global__ void __launch_bounds__(kLearnThreads, 4)
 #pragma unroll
       for (int i = 0; i < 27; ++i) v[i] = 0.0f;
     }
+    if (tile + gridDim.x < ntile) {  // the next tile's lines start their way from HBM to L2
+      int xt1, y1, z1;
+      tile_at(tile + gridDim.x, xt1, y1, z1);
+      prefetch_tile<ODD>(f, g, xt1 * kLearnThreads + 32 * warp, y1, z1, tid & 31);
+    }
     tp::pops_to_raw<float, 3>(v);
     const float drho = v[0];
     const float rho = 1.0f + drho;
-    const float irho = 1.0f / rho;
+    const float irho = __frcp_rn(rho);
     tp::Vel<float, 3> w;
     float usq = 0.0f;
 #pragma unroll
@@ -1060,7 +1099,7 @@ __global__ void __launch_bounds__(kLearnThreads, 4)
       usq += w.usq[d];
     }
     tp::raw_to_central<float, 3>(v, w.nu);
-    // features -> A1 row tid: k 0..19 features, 20..22 one (bias), 23..31 zero
+    // features -> row tid: k 0..19 features, 20..22 one (bias), 23..31 zero
     uint32_t fp[12];
     {
       float prev = 0.0f;
@@ -1081,45 +1120,46 @@ __global__ void __launch_bounds__(kLearnThreads, 4)
       fp[10] = one2;
       fp[11] = one0;
     }
-    put8(sm.a1, kK1, tid, 0, make_uint4(fp[0], fp[1], fp[2], fp[3]));
-    put8(sm.a1, kK1, tid, 1, make_uint4(fp[4], fp[5], fp[6], fp[7]));
-    put8(sm.a1, kK1, tid, 2, make_uint4(fp[8], fp[9], fp[10], fp[11]));
+    put8(sm.a, kK2, tid, 0, make_uint4(fp[0], fp[1], fp[2], fp[3]));
+    put8(sm.a, kK2, tid, 1, make_uint4(fp[4], fp[5], fp[6], fp[7]));
+    put8(sm.a, kK2, tid, 2, make_uint4(fp[8], fp[9], fp[10], fp[11]));
+    put8(sm.a, kK2, tid, 3, make_uint4(0u, 0u, 0u, 0u));
     tc05::fence_proxy_async();
     tc05::fence_before();
     if (__syncthreads_or(bad)) break;
     tc05::fence_after();
     // layer 1
-    if (tid == 0) issue_layer(tmem, sm.a1, sm.w + kB1, kK1, id64, &sm.mbar);
+    if (tid == 0) issue_layer(tmem, sm.a, sm.w + kB1, kK1, id64, &sm.mbar);
     bad |= !tc05::mbar_wait(&sm.mbar, phase, kWaitPolls);
     phase ^= 1u;
     tc05::fence_after();
-    if (!bad) relu_to_tile(trow, sm.a2, tid);
+    if (!bad) relu_to_tile(trow, sm.a, tid);
     tc05::fence_proxy_async();
     tc05::fence_before();
     if (__syncthreads_or(bad)) break;
     tc05::fence_after();
     // layer 2
-    if (tid == 0) issue_layer(tmem, sm.a2, sm.w + kB2, kK2, id64, &sm.mbar);
+    if (tid == 0) issue_layer(tmem, sm.a, sm.w + kB2, kK2, id64, &sm.mbar);
     bad |= !tc05::mbar_wait(&sm.mbar, phase, kWaitPolls);
     phase ^= 1u;
     tc05::fence_after();
-    if (!bad) relu_to_tile(trow, sm.a2, tid);
+    if (!bad) relu_to_tile(trow, sm.a, tid);
     tc05::fence_proxy_async();
     tc05::fence_before();
     if (__syncthreads_or(bad)) break;
     tc05::fence_after();
-    // layer 3 -> columns 64..79
-    if (tid == 0) issue_layer(tmem + 64, sm.a2, sm.w + kB3, kK2, id16, &sm.mbar);
+    // layer 3 -> columns 0..15
+    if (tid == 0) issue_layer(tmem, sm.a, sm.w + kB3, kK2, id16, &sm.mbar);
     bad |= !tc05::mbar_wait(&sm.mbar, phase, kWaitPolls);
     phase ^= 1u;
     tc05::fence_after();
     float zo[16];
-    if (!bad) tc05::ld16(trow + 64, zo);
-    tc05::fence_before();
-    if (__syncthreads_or(bad)) break;
+    if (!bad) tc05::ld16(trow, zo);
+    // No barrier here: every thread has seen layer 3 complete, so the tile may be written
+    // again, and the barrier before the next layer 1 orders the accumulators' reads.
     float cr[kOut];
 #pragma unroll
-    for (int c = 0; c < kOut; ++c) cr[c] = fmaf(span, 1.0f / (1.0f + __expf(-zo[c])), lo);
+    for (int c = 0; c < kOut; ++c) cr[c] = fmaf(span, __frcp_rn(1.0f + __expf(-zo[c])), lo);
     // relax: order 2 at omega_2, orders 3..6 at the class rates
 #pragma unroll
     for (int a = 0; a < 27; ++a) {
@@ -1130,14 +1170,14 @@ __global__ void __launch_bounds__(kLearnThreads, 4)
     }
     tp::central_to_raw<float, 3>(v, w.u);
     tp::raw_to_pops<float, 3>(v);
-    if (active) {
+    if (active && !bad) {
       if (!(rho > 0.0f && usq < 1.0f)) atomicOr(status, 1);
       // even sweep: population i to slot (x, opp(i)); odd sweep: to slot (x + e_i, i)
       const tp::NodeAddr<3, ODD> A(g, xc, y, z);
       tp::node_store<3, LBM_F32, ODD>(f, g, A, v);
     }
   }
-  if (bad) {
+  if (__syncthreads_or(bad)) {
     // a wait gave up: report it, give in-flight MMAs a bounded chance to finish
     if (tid == 0) atomicOr(status, 2);
     tc05::mbar_wait(&sm.mbar, phase, kWaitPolls);
@@ -1178,11 +1218,9 @@ static cudaError_t closure_sweep_tc(Sim* s, int odd, const void* img, const floa
   }
   float* f = static_cast<float*>(s->pop);
   const unsigned char* w = static_cast<const unsigned char*>(img) + kTcImageOffset;
-  if (odd)
-    learned_tc_kernel<true><<<blocks, kLearnThreads, smem, s->stream>>>(f, g, s->rates, w, norm, status_word(s));
-  else
-    learned_tc_kernel<false><<<blocks, kLearnThreads, smem, s->stream>>>(f, g, s->rates, w, norm, status_word(s));
-  return cudaGetLastError();
+  return launch_chained(odd ? learned_tc_kernel<true> : learned_tc_kernel<false>, dim3((unsigned)blocks),
+                        dim3(kLearnThreads), smem, s->stream, f, g, s->rates, w, norm, status_word(s),
+                        row_length((s->nx + kLearnThreads - 1) / kLearnThreads), row_length(s->ny));
 }
 
 cudaError_t closure_sweep(Sim* s, int odd, const void* img, const float* norm) {
@@ -1195,7 +1233,7 @@ cudaError_t closure_sweep(Sim* s, int odd, const void* img, const float* norm) {
   const int64_t cap = (int64_t)sms * 8;
   const unsigned blocks = (unsigned)(ntile < cap ? ntile : cap);
   if (closure_uses_tcgen05()) {
-    const int64_t cap_tc = (int64_t)sms * 4;  // resident blocks: 4 x 128 tensor-memory columns per SM
+    const int64_t cap_tc = (int64_t)sms * kTcBlocks;  // resident blocks
     return closure_sweep_tc(s, odd, img, norm, (int)(ntile < cap_tc ? ntile : cap_tc));
   }
   float* f = static_cast<float*>(s->pop);

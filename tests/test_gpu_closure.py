@@ -275,6 +275,29 @@ def test_constant_network_sweep_equals_plain_sweep(lbm, dims, mma_kind):
     assert b.status() == 0
 
 
+@pytest.mark.parametrize("dims,reps", [((130, 7, 5), (3, 4)), ((64, 16, 10), (3, 2))])
+def test_learned_sweep_of_a_periodic_pattern_repeats_bit_for_bit(lbm, dims, reps):
+    """A grid of copies of a small one in y and z, with more tiles than resident blocks, holds
+    the small grid's populations bit for bit: a node's update is a function of its own 27
+    values alone.  One and two tiles per row, the second with 2 nodes."""
+    def copies(a):  # (.., N) -> the larger grid
+        b = np.asarray(a).reshape(a.shape[:-1] + (dims[2], dims[1], dims[0]))
+        return np.tile(b, (1,) * (b.ndim - 3) + (reps[1], reps[0], 1)).reshape(a.shape[:-1] + (-1,))
+
+    rho, u = inputs.random_noise(dims, seed=57, du=0.04, drho=0.02)
+    P = _dev(_bf16(OC.init_params(58) * 1.5))
+    out = []
+    for d, r, v in ((dims, rho, u), ((dims[0], dims[1] * reps[0], dims[2] * reps[1]), copies(rho), copies(u))):
+        sim = lbm.Simulation("D3Q27", d, [0.6, 0.9, 0.7, 1.1, 0.8], storage="f32")
+        sim.init_fields(r, v)
+        sim.set_closure(P, _dev(ID_NORM))
+        sim.step(5)
+        assert sim.status() == 0
+        out.append(sim.populations())
+        sim.close()
+    assert np.array_equal(copies(out[0]), out[1])
+
+
 @pytest.mark.parametrize("dims,pre,lo,hi", [((20, 12, 10), 2, 0.0, 2.0), ((130, 4, 3), 3, 0.0, 2.0),
                                             ((20, 12, 10), 3, 0.5, 1.9)])
 def test_learned_sweep_matches_oracle_learned_step(lbm, dims, pre, lo, hi, mma_kind):
