@@ -330,7 +330,7 @@ int64_t lbm_step_count(lbm_handle h);
  * the range the collision is defined on: rho <= 0 or |u|^2 >= 1 in lattice
  * units on D2Q9 / D3Q27; rho <= 0, theta <= 0 or |u|^2 >= 4 in Hermite units on
  * D2Q37; or any NaN.  LBM_ETIMEOUT reports a bounded device wait that gave up
- * (the learned sweep's wait for tensor-core completion). */
+ * (the learned sweep's for tensor-core completion, the multi-step and batch sweeps'). */
 int lbm_status(lbm_handle h);
 
 /* ---- Batches of independent runs ----------------------------------------

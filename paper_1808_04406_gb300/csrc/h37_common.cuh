@@ -171,11 +171,6 @@ __device__ __forceinline__ void dot2_add_split(float& s, float& c, float x, floa
   s = t;
   c = c + __fmaf_rn(x, hl, __fmaf_rn(x, hh, -p) + es);
 }
-// s + c += x h, h given in FP64 (a compile-time constant here) and split into hi + lo
-__device__ __forceinline__ void dot2_add(float& s, float& c, float x, double h) {
-  const float hh = (float)h;
-  dot2_add_split(s, c, x, hh, (float)(h - (double)hh));
-}
 // a + b = s + e exactly
 __device__ __forceinline__ float two_sum_err(float a, float b, float s) {
   const float z = s - a;
@@ -407,18 +402,6 @@ __device__ __forceinline__ typename Store<S>::calc decode(typename Store<S>::typ
     return __bfloat162float(s) * (float)w_of(i);
   }
 }
-// Stochastically rounded encode (FP16 / BF16; the other types round as encode).
-template <int S>
-__device__ __forceinline__ typename Store<S>::type encode_sr(typename Store<S>::calc v, int i, uint32_t r) {
-  if constexpr (S == LBM_F64 || S == LBM_F32) {
-    return v;
-  } else if constexpr (S == LBM_F16) {
-    return __float2half_rz(dither(v * (float)(1.0 / w_of(i)), r, 13));
-  } else {
-    return __float2bfloat16_rz(dither(v * (float)(1.0 / w_of(i)), r, 16));
-  }
-}
-
 template <int S>
 __device__ __forceinline__ typename Store<S>::type encode(typename Store<S>::calc v, int i) {
   if constexpr (S == LBM_F64 || S == LBM_F32) {

@@ -14,7 +14,8 @@
 // an update is straight-line code, 96 KB of it for the FP32 sweep with
 // compensated table sums, whose warps waited for instructions 78 % of the time).
 // Microseconds a step, before and after: thermal FP16 1024^2 38.2 and 31.9, FP32
-// (correctly rounded) 512^2 66.5 and 20.3, 128^2 14.3 and 6.1.
+// (correctly rounded) 512^2 66.5 and 20.3, 128^2 14.3 and 6.1 (27.6, 18.2 and 4.0 since
+// the steps are chained launches and the pair sweep runs at 4 blocks per SM).
 //
 // 16-bit storage holds f_i / w_i: the weights then go into the row constants on
 // the way in (no extra operation for a row, five for the middle one), and P(e_i)

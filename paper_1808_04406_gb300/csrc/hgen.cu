@@ -217,7 +217,8 @@ __global__ void __launch_bounds__(kHgThreads)
 // sums of even and odd parity in x and y: with 37 velocities and N = 4 that takes
 // 180 FP64 operations in and 181 out, against 555 each way through the dense
 // tables, which bound this kernel (FP64 runs at 1 / 76 of the FP32 rate).
-// Shear wave on 80^2, rule E9-A, FP64: 48.2 -> 24.6 us a step (of which 18 are the FP64 pipe: one warp on each of
+// Shear wave on 80^2, rule E9-A, FP64: 48.2 -> 24.6 us a step (23.4 with
+// chained launches; 18 of them are the FP64 pipe: one warp on each of
 // 200 of the 608 SM partitions, 64 cycles per FP64 warp instruction).
 template <typename T, int NA, int NQ>
 struct Orbits {

@@ -20,7 +20,6 @@ constexpr size_t kWsStatus = 0;            // int32 status word (+ padding)
 constexpr size_t kWsResult = 256;          // 32 doubles of reduction results
 constexpr size_t kWsPartials = 512;        // kRedBlocks x 8 doubles of block partials
 constexpr int kRedBlocks = 1216;           // 8 x 152 SMs
-constexpr int kRedThreads = 256;
 constexpr int kMaxHistory = 4096;         // records of lbm_mode_history
 constexpr size_t kWsHistory = kWsPartials + (size_t)kRedBlocks * 8 * sizeof(double);
 constexpr size_t kWsFit = kWsHistory + (size_t)kMaxHistory * 2 * sizeof(double);  // 4 + 2n doubles

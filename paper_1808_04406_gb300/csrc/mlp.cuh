@@ -38,20 +38,12 @@ struct FwdW {
 };
 static_assert(sizeof(FwdW) % 16 == 0, "FwdW is copied in 16-byte units");
 
-struct BwdW {
-  __nv_bfloat16 w2s[kH][kLdH];
-  __nv_bfloat16 w3s[kH][kOutPad];
-};
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t d;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
   return d;
 }
 __device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
-__device__ __forceinline__ uint32_t pack2h(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
 
 __device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
@@ -81,17 +73,6 @@ __device__ __forceinline__ void load_fwd(const float* __restrict__ P, FwdW& s) {
     s.b2[i] = P[kOffB2 + i];
   }
   for (int i = threadIdx.x; i < kOutPad; i += blockDim.x) s.b3[i] = i < kOut ? P[kOffB3 + i] : 0.0f;
-}
-
-__device__ __forceinline__ void load_bwd(const float* __restrict__ P, BwdW& s) {
-  for (int i = threadIdx.x; i < kH * kLdH; i += blockDim.x) {
-    const int a = i / kLdH, b = i % kLdH;
-    s.w2s[a][b] = __float2bfloat16_rn(b < kH ? P[kOffW2 + a * kH + b] : 0.0f);
-  }
-  for (int i = threadIdx.x; i < kH * kOutPad; i += blockDim.x) {
-    const int k = i / kOutPad, n = i % kOutPad;
-    s.w3s[k][n] = __float2bfloat16_rn(n < kOut ? P[kOffW3 + k * kOut + n] : 0.0f);
-  }
 }
 
 // Copy a prepared forward image (global, 16-byte aligned) into shared memory.

@@ -58,9 +58,10 @@ __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks)
 // collided, so their latency overlaps the collision instead of stalling it.
 // (AA slots belong to one node per sweep, so loading the next pair before the
 // current one is stored is race-free.)  The node arithmetic is that of
-// tp_pair_kernel, and so are the results, bit for bit.  At 4 blocks per SM the
-// compiler keeps it within 128 registers without spills (the one-pair kernel
-// needs 158-164 and so runs at 3).
+// tp_pair_kernel, and so are the results, bit for bit.  At 4 blocks per SM
+// the compiler keeps it within 128 registers (16 bytes spilled in the odd sweep, which
+// executes 1112 instructions per pair against the even one's 782: addresses of shifted
+// slots, and 2-byte accesses for e_x = 0).
 //
 // The walk is 8 planes, or fewer where that would leave less than 900 blocks, one
 // and a half waves of 608 (FP16, us a step, walks of 8 and of 1: 64^3 10.9 and 7.7,
