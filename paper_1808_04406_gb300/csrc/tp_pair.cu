@@ -98,22 +98,45 @@ __global__ void __launch_bounds__(kPairThreads, kZRunMinBlocks)
   if (!ok) atomicOr(status, 1);
 }
 
+// The five sums of a warp, each by the tree of offsets 16, 8, 4, 2, 1.  Where two values
+// are left to reduce, the halves of the warp take one each (addition commutes, so every
+// sum is that of the five separate trees, bit for bit): 8 shuffles instead of 25.
+// A D3Q27 FP32 run of 20 steps with totals on 128^3, fields in and out: 2636 us with 25
+// shuffles in plain launches at 3 blocks per SM, 2186 so.  (One tree for 4 planes of a
+// thread takes 2062, but other nodes of a warp meet in FP32: totals 2e-8 apart.)
+__device__ __forceinline__ float fold2(float a, float b, int o, int lane) {
+  const bool up = (lane & o) != 0;
+  return (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, o);
+}
+__device__ __forceinline__ float fold1(float a, int o) { return a + __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ void write_partials(const float (&acc)[5], float* __restrict__ partials) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  float s = fold2(fold2(acc[0], acc[1], 16, lane), fold2(acc[2], acc[3], 16, lane), 8, lane);
+  s = fold2(s, fold1(fold1(acc[4], 16), 8), 4, lane);
+  s = fold1(fold1(s, 2), 1);
+  // sum k now sits in lane 0, 16, 8, 24, 4
+  const int k = lane & 4 ? 4 : (lane >> 4) + ((lane & 8) >> 2);
+  if ((lane & 3) == 0 && (k < 4 || lane == 4)) {
+    const size_t b = (size_t)blockIdx.x + (size_t)gridDim.x * ((size_t)blockIdx.y + (size_t)gridDim.y * blockIdx.z);
+    partials[(b * (kPairThreads / 32) + (size_t)wid) * 8 + k] = s;
+  }
+}
+
 // The plane-walking sweep with the totals of the consumed state, as
 // tp_pair_totals_kernel computes them per node; each thread adds its nodes of
 // all its planes in FP32 before the warp's shuffle tree, so there is one
-// partial per warp of this grid (tp_pair_warps).
+// partial per warp of this grid (tp_pair_warps).  Walks of kZRun planes on every grid,
+// and threads along the rows (see tp_pair_totals_kernel).
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kPairThreads, 3)  // the running totals need more than 128 registers
     tp_pair_zrun_totals_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r,
-                               int* __restrict__ status, float* __restrict__ partials, RowLength row, int z0,
-                               int z1, int run) {
-  int xp, y;
-  const bool in = row_of(blockIdx.x * blockDim.x + threadIdx.x, row, g.ny, xp, y);
+                               int* __restrict__ status, float* __restrict__ partials, int z0, int z1) {
+  const int xp = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   chain_wait();
-  if (in) {
-    const int zb = z0 + (int)blockIdx.z * run;
-    const int ze = zb + run < z1 ? zb + run : z1;
+  if (xp < (g.nx >> 1)) {
+    const int zb = z0 + (int)blockIdx.z * kZRun;
+    const int ze = zb + kZRun < z1 ? zb + kZRun : z1;
     f2 om[7];
 #pragma unroll
     for (int n = 0; n < 7; ++n) om[n] = cst<f2>(r.w[n]);
@@ -142,17 +165,7 @@ __global__ void __launch_bounds__(kPairThreads, 3)  // the running totals need m
     }
     if (!ok) atomicOr(status, 1);
   }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
-  if (lane == 0) {
-    const size_t b = (size_t)blockIdx.x + (size_t)gridDim.x * ((size_t)blockIdx.y + (size_t)gridDim.y * blockIdx.z);
-    const size_t w = b * (kPairThreads / 32) + (size_t)wid;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) partials[w * 8 + k] = acc[k];
-  }
+  write_partials(acc, partials);
 }
 
 // The same sweep, which also writes per block the FP64 totals of the state it
@@ -164,58 +177,40 @@ __global__ void __launch_bounds__(kPairThreads, 3)  // the running totals need m
 // this GPU: per-node FP64 sums would double the sweep's time; and no block
 // barrier holds finished warps back.)
 //
-// On D3Q27 a thread adds up the pairs of up to kTotalsRun planes first: fewer
-// shuffles (a seventh of the kernel's instructions with one plane) and fewer
-// partials.
-constexpr int kTotalsRun = 4;
+// Threads run along the rows here, and a warp's 64 nodes are of one row: which nodes a
+// warp adds up in FP32 decides the last bits of the totals.
 template <int D, int S, bool ODD>
 __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks)
     tp_pair_totals_kernel(typename PairIO<S>::E* __restrict__ f, tp::Grid g, Rates r, int* __restrict__ status,
-                          float* __restrict__ partials, RowLength row, int z0, int z1, int run) {
-  int xp, y;
-  const bool in = row_of(blockIdx.x * blockDim.x + threadIdx.x, row, g.ny, xp, y);
+                          float* __restrict__ partials, int z0) {
+  int xp = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z + z0;
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   chain_wait();
-  if (in) {
+  if (xp < (g.nx >> 1)) {
     f2 om[2 * D + 1];
 #pragma unroll
     for (int n = 0; n <= 2 * D; ++n) om[n] = cst<f2>(r.w[n]);
-    const int zb = z0 + (int)blockIdx.z * run, ze = zb + run < z1 ? zb + run : z1;
-    bool ok = true;
-#pragma unroll 1
-    for (int z = zb; z < ze; ++z) {
-      f2 v[tp::qof<D>()];
-      tp::pair_load<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
-      if constexpr (D == 3) forget(xp, y, z);
-      tp::NodeMoments<f2, D> m;
-      ok = tp::collide<f2, D, true>(v, om, &m) && ok;
-      tp::pair_store<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
-      float d0, d1, jj0 = 0.0f, jj1 = 0.0f;
-      unpack2(m.drho, d0, d1);
-      acc[0] += d0 + d1;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        float j0, j1;
-        unpack2(m.j[d], j0, j1);
-        acc[1 + d] += j0 + j1;
-        jj0 += j0 * j0;
-        jj1 += j1 * j1;
-      }
-      acc[4] += __fdividef(0.5f * jj0, 1.0f + d0) + __fdividef(0.5f * jj1, 1.0f + d1);
-    }
+    f2 v[tp::qof<D>()];
+    tp::pair_load<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
+    if constexpr (D == 3) forget(xp, y, z);
+    tp::NodeMoments<f2, D> m;
+    const bool ok = tp::collide<f2, D, true>(v, om, &m);
+    tp::pair_store<D, S, ODD>(f, g, tp::PairAddr<D, ODD>(g, xp, y, z), v);
     if (!ok) atomicOr(status, 1);
+    float d0, d1, jj0 = 0.0f, jj1 = 0.0f;
+    unpack2(m.drho, d0, d1);
+    acc[0] = d0 + d1;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      float j0, j1;
+      unpack2(m.j[d], j0, j1);
+      acc[1 + d] = j0 + j1;
+      jj0 += j0 * j0;
+      jj1 += j1 * j1;
+    }
+    acc[4] = __fdividef(0.5f * jj0, 1.0f + d0) + __fdividef(0.5f * jj1, 1.0f + d1);
   }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
-  if (lane == 0) {
-    const size_t b = (size_t)blockIdx.x + (size_t)gridDim.x * ((size_t)blockIdx.y + (size_t)gridDim.y * blockIdx.z);
-    const size_t w = b * (kPairThreads / 32) + (size_t)wid;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) partials[w * 8 + k] = acc[k];
-  }
+  write_partials(acc, partials);
 }
 
 // LBM_TP_ZRUN=0 keeps one pair per thread for 16-bit D3Q27 (read at every
@@ -229,9 +224,9 @@ inline unsigned plane_blocks(const Sim* s) {
   return (unsigned)((s->nx / 2 * s->ny + kPairThreads - 1) / kPairThreads);
 }
 
-// Planes per thread, at most `longest`.
-inline int walk_of(const Sim* s, int longest) {
-  int run = longest;
+// Planes per thread.
+inline int walk_of(const Sim* s) {
+  int run = kZRun;
   while (run > 1 && (int64_t)plane_blocks(s) * ((active_nz(s) + run - 1) / run) < kZRunMinGrid) run /= 2;
   return run;
 }
@@ -241,7 +236,7 @@ cudaError_t launch_zrun(Sim* s, int odd) {
   using E = typename PairIO<S>::E;
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
   const int64_t nzs = active_nz(s);
-  const int run = walk_of(s, kZRun);
+  const int run = walk_of(s);
   dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
   const int z0 = (int)active_z0(s), z1 = (int)(active_z0(s) + nzs);
   E* f = static_cast<E*>(s->pop);
@@ -264,34 +259,27 @@ cudaError_t launch(Sim* s, int odd) {
                         s->rates, status_word(s), row_length(s->nx / 2), z0);
 }
 
-template <int S>
-cudaError_t launch_zrun_totals(Sim* s, int odd, float* partials) {
-  using E = typename PairIO<S>::E;
-  tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
-  const int64_t nzs = active_nz(s);
-  const int run = walk_of(s, kZRun);
-  dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
-  const int z0 = (int)active_z0(s), z1 = (int)(active_z0(s) + nzs);
-  E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? tp_pair_zrun_totals_kernel<S, true> : tp_pair_zrun_totals_kernel<S, false>, grid,
-                        dim3(kPairThreads), 0, s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
+// blocks of the totals sweeps: rows, each of one or more blocks, and planes or walks of kZRun
+inline dim3 totals_grid(const Sim* s) {
+  const int64_t run = s->D == 3 && s->storage != LBM_F32 && zrun_enabled() ? kZRun : 1;
+  return dim3((unsigned)((s->nx / 2 + kPairThreads - 1) / kPairThreads), (unsigned)s->ny,
+              (unsigned)((active_nz(s) + run - 1) / run));
 }
 
 template <int D, int S>
 cudaError_t launch_totals(Sim* s, int odd, float* partials) {
   using E = typename PairIO<S>::E;
-  if constexpr (D == 3 && S != LBM_F32) {
-    if (zrun_enabled()) return launch_zrun_totals<S>(s, odd, partials);
-  }
   tp::Grid g{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
-  const int64_t nzs = active_nz(s);
-  dim3 block(kPairThreads);
-  const int run = D == 2 ? 1 : walk_of(s, kTotalsRun);
-  dim3 grid(plane_blocks(s), 1, (unsigned)((nzs + run - 1) / run));
-  const int z0 = (int)active_z0(s), z1 = (int)(z0 + nzs);
+  const int z0 = (int)active_z0(s), z1 = (int)(z0 + active_nz(s));
   E* f = static_cast<E*>(s->pop);
-  return launch_chained(odd ? tp_pair_totals_kernel<D, S, true> : tp_pair_totals_kernel<D, S, false>, grid, block, 0,
-                        s->stream, f, g, s->rates, status_word(s), partials, row_length(s->nx / 2), z0, z1, run);
+  if constexpr (D == 3 && S != LBM_F32) {
+    if (zrun_enabled())
+      return launch_chained(odd ? tp_pair_zrun_totals_kernel<S, true> : tp_pair_zrun_totals_kernel<S, false>,
+                            totals_grid(s), dim3(kPairThreads), 0, s->stream, f, g, s->rates, status_word(s), partials,
+                            z0, z1);
+  }
+  return launch_chained(odd ? tp_pair_totals_kernel<D, S, true> : tp_pair_totals_kernel<D, S, false>, totals_grid(s),
+                        dim3(kPairThreads), 0, s->stream, f, g, s->rates, status_word(s), partials, z0);
 }
 
 template <int D>
@@ -327,9 +315,8 @@ cudaError_t tp_launch_pair_sweep(Sim* s, int odd) {
 }
 
 int64_t tp_pair_warps(const Sim* s) {
-  const int64_t nz = active_nz(s);
-  const int run = s->D == 2 ? 1 : walk_of(s, s->storage != LBM_F32 && zrun_enabled() ? kZRun : kTotalsRun);
-  return (int64_t)plane_blocks(s) * ((nz + run - 1) / run) * (kPairThreads / 32);
+  const dim3 b = totals_grid(s);
+  return (int64_t)b.x * b.y * b.z * (kPairThreads / 32);
 }
 
 cudaError_t tp_launch_pair_sweep_totals(Sim* s, int odd, float* partials) {
