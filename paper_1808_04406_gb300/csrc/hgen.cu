@@ -577,6 +577,181 @@ __global__ void __launch_bounds__(kHgThreads)
   orbit_store<ODD>(f, g, rule, x, y, v);
 }
 
+// The FP64 sweep with two threads per node, for grids that leave SM partitions empty: a
+// partition issues one FP64 warp instruction per 64 cycles however few of its lanes are
+// active, so more warps of shorter streams are faster while partitions are free.  The
+// first thread of a node takes the x pairs and half of the quadruples; the second takes
+// the y pairs and the other half, with x and y exchanged, so that both run the same
+// code.  Each adds the other's sums to its own (102 FP64 operations in and 91 out,
+// against 180 and 181); both compute the collision, from the same bits.  Shear wave on
+// 80^2, rule E9-A, with its amplitude records: 23.4 -> 19.3 us a step.
+template <int NA, int NH>
+struct HalfOrbits {
+  struct Pair {
+    int i[2], a;         // +, -; |e|
+    double c[5], v[5];   // a^n, w a^n
+  } p[NA];
+  struct Quad {
+    int i[4], a, b;         // (a, b), (-a, b), (a, -b), (-a, -b); a = 0: none
+    double c[15], v[15];    // a^p b^q, w a^p b^q
+  } q[NH];
+};
+template <int NA, int NH>
+struct HalfRule {
+  HalfOrbits<NA, NH> half[2];
+  HMap map;
+  int rest;
+  double w0;
+};
+
+template <int NA, int NQ>
+void split_orbits(const OrbitRule<double, NA, NQ>& r, HalfRule<NA, (NQ + 1) / 2>* out) {
+  const auto& o = r.o;
+  *out = HalfRule<NA, (NQ + 1) / 2>{};
+  out->map = r.map;
+  out->rest = o.rest;
+  out->w0 = o.w0;
+  for (int h = 0; h < 2; ++h) {
+    for (int k = 0; k < NA; ++k) {
+      auto& p = out->half[h].p[k];
+      p.i[0] = h ? o.yp[k] : o.xp[k];
+      p.i[1] = h ? o.ym[k] : o.xm[k];
+      p.a = o.da[k];
+      for (int n = 0; n < 5; ++n) {
+        p.c[n] = n ? p.c[n - 1] * p.a : 1.0;
+        p.v[n] = o.pw[k] * p.c[n];
+      }
+    }
+    for (int k = 0; k < (NQ + 1) / 2; ++k) {
+      auto& q = out->half[h].q[k];
+      const int j = 2 * k + h;
+      if (j >= NQ) {
+        for (int& i : q.i) i = o.rest;
+        continue;
+      }
+      q.i[0] = o.pp[j];
+      q.i[1] = h ? o.pm[j] : o.mp[j];
+      q.i[2] = h ? o.mp[j] : o.pm[j];
+      q.i[3] = o.mm[j];
+      q.a = h ? o.qb[j] : o.qa[j];
+      q.b = h ? o.qa[j] : o.qb[j];
+      for (int c = 0; c < 15; ++c) {
+        q.c[c] = 1.0;  // small integers: exact
+        for (int n = 0; n < h37::cp(c); ++n) q.c[c] *= q.a;
+        for (int n = 0; n < h37::cq(c); ++n) q.c[c] *= q.b;
+        q.v[c] = o.qw[j] * q.c[c];
+      }
+    }
+  }
+}
+
+template <int NC, int NA, int NH, bool ODD>
+__global__ void __launch_bounds__(32)
+    hgen_half_kernel(double* __restrict__ f, HGrid g, const __grid_constant__ HalfRule<NA, NH> rule,
+                     const __grid_constant__ h37::MomentModel<double> m, int* __restrict__ status) {
+  using h37::cidx;
+  using h37::cp;
+  using h37::cq;
+  const uint32_t id = blockIdx.x * 32 + threadIdx.x;
+  const int h = (int)(id & 1);
+  const HalfOrbits<NA, NH>& o = rule.half[h];
+  chain_wait();
+  const bool in = (id >> 1) < (uint32_t)g.N;
+  const uint32_t node = in ? id >> 1 : 0u;  // threads past the grid take part in the exchange
+  const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
+  auto nbr = [&](int ex, int ey) { return h ? hnbr(g, x, y, ey, ex) : hnbr(g, x, y, ex, ey); };
+  auto load = [&](int i, int ex, int ey, int opp) {
+    return ODD ? f[(size_t)opp * g.N + nbr(-ex, -ey)] : f[(size_t)i * g.N + node];
+  };
+  auto store = [&](double v, int i, int ex, int ey, int opp) {
+    if (ODD)
+      f[(size_t)i * g.N + nbr(ex, ey)] = v;
+    else
+      f[(size_t)opp * g.N + node] = v;
+  };
+  double vr = load(rule.rest, 0, 0, rule.rest), vp[NA][2], vq[NH][4];
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    vp[k][0] = load(o.p[k].i[0], o.p[k].a, 0, o.p[k].i[1]);
+    vp[k][1] = load(o.p[k].i[1], -o.p[k].a, 0, o.p[k].i[0]);
+  }
+#pragma unroll
+  for (int k = 0; k < NH; ++k) {
+    const int a = o.q[k].a, b = o.q[k].b;
+    vq[k][0] = load(o.q[k].i[0], a, b, o.q[k].i[3]);
+    vq[k][1] = load(o.q[k].i[1], -a, b, o.q[k].i[2]);
+    vq[k][2] = load(o.q[k].i[2], a, -b, o.q[k].i[1]);
+    vq[k][3] = load(o.q[k].i[3], -a, -b, o.q[k].i[0]);
+    if (a == 0) vq[k][0] = vq[k][1] = vq[k][2] = vq[k][3] = 0.0;
+  }
+  double M[NC], H[NC], inc[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) M[c] = 0.0;
+  if (h == 0) M[0] = vr;
+#pragma unroll
+  for (int k = 0; k < NH; ++k) {
+    const double s1 = vq[k][0] + vq[k][3], d1 = vq[k][0] - vq[k][3], s2 = vq[k][2] + vq[k][1], d2 = vq[k][2] - vq[k][1];
+    const double z[4] = {s1 + s2, d1 + d2, d1 - d2, s1 - s2};  // parities (even, even), (odd, even), (even, odd), (odd, odd)
+    M[0] += z[0];
+#pragma unroll
+    for (int c = 1; c < NC; ++c) M[c] = fma_(o.q[k].c[c], z[(cp(c) & 1) + 2 * (cq(c) & 1)], M[c]);
+  }
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    const double sx = vp[k][0] + vp[k][1], dx = vp[k][0] - vp[k][1];
+    M[0] += sx;
+#pragma unroll
+    for (int n = 1; n <= (NC == 15 ? 4 : 3); ++n) M[cidx(n, 0)] = fma_(o.p[k].c[n], n & 1 ? dx : sx, M[cidx(n, 0)]);
+  }
+  {
+    double other[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) other[c] = __shfl_xor_sync(0xffffffffu, M[cidx(cq(c), cp(c))], 1);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) M[c] += other[c];
+  }
+  h37::to_basis<double, NC>(M, H, m);
+  const bool ok = h37::moment_increments<double, NC>(H, inc, m);
+  // the second thread's increments are the first's: its own may differ in the last bits
+#pragma unroll
+  for (int c = 3; c < NC; ++c) {
+    const double first = __shfl_sync(0xffffffffu, inc[c], threadIdx.x & 30);
+    H[c] = first;
+  }
+#pragma unroll
+  for (int c = 3; c < NC; ++c) M[c] += h ? H[cidx(cq(c), cp(c))] : H[c];
+  h37::to_polynomial<double, NC>(M, rule.map);
+  if (!in) return;
+  if (!ok) atomicOr(status, 1);
+  if (h == 0) store(rule.w0 * M[0], rule.rest, 0, 0, rule.rest);
+#pragma unroll
+  for (int k = 0; k < NA; ++k) {
+    const auto& p = o.p[k];
+    double e = fma_(p.v[2], M[cidx(2, 0)], p.v[0] * M[0]);
+    if constexpr (NC == 15) e = fma_(p.v[4], M[cidx(4, 0)], e);
+    const double od = fma_(p.v[3], M[cidx(3, 0)], p.v[1] * M[cidx(1, 0)]);
+    store(e + od, p.i[0], p.a, 0, p.i[1]);
+    store(e - od, p.i[1], -p.a, 0, p.i[0]);
+  }
+#pragma unroll
+  for (int k = 0; k < NH; ++k) {
+    const auto& q = o.q[k];
+    double z[4] = {q.v[0] * M[0], q.v[1] * M[1], q.v[2] * M[2], q.v[cidx(1, 1)] * M[cidx(1, 1)]};
+#pragma unroll
+    for (int c = 3; c < NC; ++c) {
+      if (c == cidx(1, 1)) continue;
+      double& t = z[(cp(c) & 1) + 2 * (cq(c) & 1)];
+      t = fma_(q.v[c], M[c], t);
+    }
+    const double s1 = z[0] + z[3], s2 = z[0] - z[3], t1 = z[1] + z[2], t2 = z[1] - z[2];
+    if (q.a == 0) continue;
+    store(s1 + t1, q.i[0], q.a, q.b, q.i[3]);
+    store(s1 - t1, q.i[3], -q.a, -q.b, q.i[0]);
+    store(s2 + t2, q.i[2], q.a, -q.b, q.i[1]);
+    store(s2 - t2, q.i[1], -q.a, q.b, q.i[2]);
+  }
+}
+
 __device__ __forceinline__ void hxy_of(const HGrid& g, int64_t n, int& x, int& y) {
   const uint32_t nn = (uint32_t)n, nx = (uint32_t)g.nx;
   y = (int)(nn / nx);
@@ -806,6 +981,19 @@ cudaError_t orbit_sweep(Sim* s, int odd, bool* taken) {
   while (t > 32 && s->N < (int64_t)t * 2 * 152) t /= 2;
   const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   T* f = static_cast<T*>(s->pop);
+  if constexpr (S == LBM_F64) {
+    // two threads per node while that leaves at most one warp per SM partition: beyond, a
+    // partition would issue two shorter streams instead of one (us a step, one thread and
+    // two: 80^2 22.3 and 18.2, 64 x 152 22.3 and 18.1, 100^2 22.4 and 23.9, 139^2 25.4 and 33.1)
+    if (s->N <= (int64_t)4 * 152 * 16) {
+      HalfRule<NA, (NQ + 1) / 2> half;
+      split_orbits(rule, &half);
+      constexpr int NH = (NQ + 1) / 2;
+      return launch_chained(odd ? hgen_half_kernel<NC, NA, NH, true> : hgen_half_kernel<NC, NA, NH, false>,
+                            dim3((unsigned)((2 * s->N + 31) / 32)), dim3(32), 0, s->stream, f, hgrid(s), half,
+                            hmoment_model<T>(s), status_word(s));
+    }
+  }
   return launch_chained(odd ? hgen_orbit_kernel<T, NC, NA, NQ, true> : hgen_orbit_kernel<T, NC, NA, NQ, false>,
                         dim3(blocks), dim3(t), 0, s->stream, f, hgrid(s), rule, hmoment_model<T>(s), status_word(s));
 }

@@ -163,6 +163,35 @@ def test_shear_viscosity_from_the_device_fit(lbm, name):
 
 
 @pytest.mark.parametrize("name", ["E7-A", "E7-D", "E9-A", "E9-C"])
+@pytest.mark.parametrize("flags", ["thermal", "isothermal"])
+def test_two_threads_per_node_match_one(lbm, name, flags):
+    """FP64 grids of up to 9728 nodes give every node two threads.  A field constant in y
+    on 64 x 152 nodes (two threads, 9728) and on 64 x 153 (one) holds the same columns,
+    but for the order of summation: 5 steps within the bound of the test below."""
+    nx, taus = 64, TAUS
+    rho, u, theta = _fields((nx, 3), seed=23)
+    out = []
+    for ny in (152, 153):
+        r = np.tile(rho[:nx], ny)
+        v = np.tile(u[:, :nx], (1, ny))
+        t = np.tile(theta[:nx], ny)
+        s = lbm.HermiteSimulation(gen_rules.rule(name), (nx, ny), taus, storage="f64",
+                                  flags=lbm.LBM_THERMAL if flags == "thermal" else 0, theta_ref=1.1)
+        if flags == "thermal":
+            s.init_fields(r, v, t)
+        else:
+            s.init_fields(r, v)
+        s.step(5)
+        assert s.status() == 0
+        out.append(s.populations())
+        s.close()
+    q = out[0].shape[0]
+    a, b = (o.reshape(q, -1, nx) for o in out)
+    np.testing.assert_allclose(a[:, :2], b[:, :2], rtol=0, atol=5e-14)
+    assert np.array_equal(a, np.repeat(a[:, :1], a.shape[1], axis=1))
+
+
+@pytest.mark.parametrize("name", ["E7-A", "E7-D", "E9-A", "E9-C"])
 @pytest.mark.parametrize("storage", ["f64", "f32"])
 @pytest.mark.parametrize("dims", [(3, 3), (13, 7), (37, 263)])
 def test_orbit_sweep_matches_the_dense_tables(lbm, name, storage, dims):
