@@ -790,11 +790,11 @@ def run_batch(args):
 
 
 THERMAL_N, THERMAL_THETA0, THERMAL_PR = 1024, 1.2, 0.71
-# FP32 arithmetic of one 37-velocity thermal lattice update: 2 x 515 FFMA + 172 FADD +
-# 36 FMUL, the one-node kernel's executed counts (ncu, FP32 storage, both parities);
-# 16-bit offsets add 37 + 37 FMUL for the w_i scaling.
-H37_FLOPS_PER_LUP = 1238.0
-H37_SCALE_FLOPS = 74.0
+# FP32 arithmetic of one 37-velocity thermal lattice update, the one-node kernel's executed
+# counts (ncu, both parities): FP32 storage through the Hermite tables 2 x 515 FFMA + 172
+# FADD + 36 FMUL; 16-bit storage through raw moments 2 x 211 FFMA + 188 FADD + 75 FMUL
+# (FP64 storage takes the same steps).
+H37_FLOPS_PER_LUP = {8: 685.0, 4: 1238.0, 2: 685.0}  # by element size
 # FP32 ALU peak from unit counts: 128 FP32 FMA lanes per SM x 2 flop x SMs x SM clock.
 FP32_LANES_PER_SM = 128
 
@@ -928,7 +928,7 @@ def run_thermal(args):
            "traffic": None, "peak_kind": peak_kind, "algorithmic_bytes_per_launch": bpl * n * n}
     clocks = clk.summary()
     sm_mhz = clocks.get("sm_max_mhz") or 2070.0
-    flops = H37_FLOPS_PER_LUP + (H37_SCALE_FLOPS if esize == 2 else 0.0)
+    flops = H37_FLOPS_PER_LUP[esize]
     # the sweep issues packed FP32x2 FMAs: its peak is the packed probe's (measured in this run)
     alu_peak = measure_alu_peak("f32x2")
     alu_achieved = flops * n * n / launch / 1e12
