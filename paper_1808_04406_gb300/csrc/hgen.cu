@@ -10,8 +10,9 @@
 // Velocities crossing the C ABI are in lattice units.
 //
 // Rules that are symmetric under e_x -> -e_x and e_y -> -e_y (every minimal rule
-// is) go through hgen_orbit_kernel: raw moments of the reflection orbits.  Others,
-// and plain FP32 transforms, take the dense tables (hgen_sweep_kernel).
+// is) go, in FP64, through hgen_orbit_kernel: raw moments of the reflection orbits
+// (hgen_half_kernel on small grids).  Others, and FP32, take the dense tables
+// (hgen_sweep_kernel).
 #include <cmath>
 #include <type_traits>
 
@@ -224,7 +225,7 @@ template <typename T, int NA, int NQ>
 struct Orbits {
   int rest, xp[NA], xm[NA], yp[NA], ym[NA], pp[NQ], mp[NQ], pm[NQ], mm[NQ];  // velocity indices
   int da[NA], qa[NQ], qb[NQ];                                                // |e| of pairs, |e_x| and |e_y| of quadruples
-  T w0, pw[NA], qw[NQ];                                                      // weights (1 where a sum is weighted later)
+  T w0, pw[NA], qw[NQ];                                                      // weights
   T p1[NA], p2[NA], p3[NA], p4[NA];                                          // powers of a
   T a1[NQ], a2[NQ], a3[NQ], a4[NQ], b1[NQ], b2[NQ], b3[NQ], b4[NQ];          // a^p b^q of quadruples
   T ab[NQ], a2b[NQ], ab2[NQ], a2b2[NQ], a3b[NQ], ab3[NQ];
@@ -234,9 +235,9 @@ struct Orbits {
 };
 
 // Fills o from the rule; false if the rule lacks a reflection, has other numbers of
-// orbits, or weights that differ within an orbit.  weighted = false: weights of 1.
+// orbits, or weights that differ within an orbit.
 template <typename T, int NA, int NQ>
-bool make_orbits(const HLattice& L, bool weighted, Orbits<T, NA, NQ>* o) {
+bool make_orbits(const HLattice& L, Orbits<T, NA, NQ>* o) {
   int at[7][7];
   for (auto& r : at)
     for (int& k : r) k = -1;
@@ -246,7 +247,7 @@ bool make_orbits(const HLattice& L, bool weighted, Orbits<T, NA, NQ>* o) {
   int na = 0, nq = 0;
   o->rest = idx(0, 0);
   if (o->rest < 0) return false;
-  o->w0 = weighted ? (T)L.w[o->rest] : T(1);
+  o->w0 = (T)L.w[o->rest];
   for (int a = 1; a <= 3; ++a) {
     const int xp = idx(a, 0), xm = idx(-a, 0), yp = idx(0, a), ym = idx(0, -a);
     if (xp < 0 && xm < 0 && yp < 0 && ym < 0) continue;
@@ -256,7 +257,7 @@ bool make_orbits(const HLattice& L, bool weighted, Orbits<T, NA, NQ>* o) {
     o->yp[na] = yp;
     o->ym[na] = ym;
     o->da[na] = a;
-    const double w = weighted ? L.w[xp] : 1.0, d = a;
+    const double w = L.w[xp], d = a;
     o->pw[na] = (T)w;
     o->p1[na] = (T)d;
     o->p2[na] = (T)(d * d);
@@ -280,7 +281,7 @@ bool make_orbits(const HLattice& L, bool weighted, Orbits<T, NA, NQ>* o) {
       o->mm[k] = mm;
       o->qa[k] = a;
       o->qb[k] = b;
-      const double w = weighted ? L.w[pp] : 1.0, x = a, y = b;
+      const double w = L.w[pp], x = a, y = b;
       o->qw[k] = (T)w;
       o->a1[k] = (T)x;
       o->a2[k] = (T)(x * x);
@@ -339,7 +340,6 @@ struct OrbitValues {
   }
 };
 
-// T: the values' type (f2: hi and lo parts), R: that of the constants
 template <typename T, typename R, int NA, int NQ, int NC>
 __device__ __forceinline__ void orbit_moments(const Orbits<R, NA, NQ>& o, const OrbitValues<T, NA, NQ>& v,
                                               T (&M)[NC]) {
@@ -388,13 +388,12 @@ __device__ __forceinline__ void orbit_moments(const Orbits<R, NA, NQ>& o, const 
   }
 }
 
-// w P(e) at every velocity (P(e) where the weights of o are 1)
+// w P(e) at every velocity
 template <typename T, typename R, int NA, int NQ, int NC>
-__device__ __forceinline__ void orbit_values(const Orbits<R, NA, NQ>& o, const T (&b)[NC], OrbitValues<T, NA, NQ>& v,
-                                             bool weighted) {
+__device__ __forceinline__ void orbit_values(const Orbits<R, NA, NQ>& o, const T (&b)[NC], OrbitValues<T, NA, NQ>& v) {
   using h37::cidx;
   using h37::spread;
-  auto w0 = [&](R w, T x) { return weighted ? spread<T>(w) * x : x; };
+  auto w0 = [&](R w, T x) { return spread<T>(w) * x; };
   auto add = [&](R k, int c, T x) { return fma_(spread<T>(k), b[c], x); };
   auto mul = [&](R k, int c) { return spread<T>(k) * b[c]; };
   v.r = w0(o.w0, b[0]);
@@ -431,8 +430,7 @@ __device__ __forceinline__ void orbit_values(const Orbits<R, NA, NQ>& o, const T
   }
 }
 
-// The constants of h37::to_polynomial (FP64) and of its correctly rounded form for
-// the rule's c.
+// The constants of h37::to_polynomial for the rule's c.
 struct HMap {
   double v[13];
   __device__ __forceinline__ double ns() const { return v[0]; }
@@ -449,32 +447,11 @@ struct HMap {
   __device__ __forceinline__ double n4s() const { return v[11]; }
   __device__ __forceinline__ double n4f() const { return v[12]; }
 };
-struct HSplitMap {
-  h37::Split v[h37::kMapTerms];
-  __device__ __forceinline__ h37::Split at(int t) const { return v[t]; }
-};
 template <typename T, int NA, int NQ>
-struct HSplitWeights {
-  h37::Split w0, pw[NA], qw[NQ];
-};
-template <typename T, int NA, int NQ>
-struct OrbitRule;
-template <int NA, int NQ>
-struct OrbitRule<double, NA, NQ> {
-  Orbits<double, NA, NQ> o;
+struct OrbitRule {
+  Orbits<T, NA, NQ> o;
   HMap map;
 };
-template <int NA, int NQ>
-struct OrbitRule<float, NA, NQ> {
-  Orbits<float, NA, NQ> o;
-  HSplitMap map;
-  HSplitWeights<float, NA, NQ> w;
-};
-
-// sums of |e_x^p e_y^q| over any 37 velocities with |e| <= 3 (p + q = 4: at most
-// 36 * 81), and over p + q <= 4 at (3, 3) (547), as powers of two
-constexpr int kOrbitMomentBits = 12;
-constexpr int kOrbitPolynomialBits = 10;
 
 template <int NA, int NQ, int NC>
 __device__ __forceinline__ bool orbit_update(const OrbitRule<double, NA, NQ>& rule, OrbitValues<double, NA, NQ>& v,
@@ -486,59 +463,7 @@ __device__ __forceinline__ bool orbit_update(const OrbitRule<double, NA, NQ>& ru
 #pragma unroll
   for (int k = 3; k < NC; ++k) M[k] += inc[k];
   h37::to_polynomial<double, NC>(M, rule.map);
-  orbit_values<double>(rule.o, M, v, true);
-  return ok;
-}
-
-// FP32, correctly rounded (see h37_moments.cuh)
-template <int NA, int NQ, int NC>
-__device__ __forceinline__ bool orbit_update(const OrbitRule<float, NA, NQ>& rule, OrbitValues<float, NA, NQ>& v,
-                                             const h37::MomentModel<float>& m) {
-  float mx = 0.f;
-  v.each(rule.o, [&](float& x, int, int, int, int) { mx = fmaxf(mx, fabsf(x)); });
-  const float sigma = h37::cut_at(mx, kOrbitMomentBits);
-  OrbitValues<f2, NA, NQ> x;
-  x.r = h37::cut(v.r, sigma);
-#pragma unroll
-  for (int k = 0; k < NA; ++k) {
-    x.xp[k] = h37::cut(v.xp[k], sigma);
-    x.xm[k] = h37::cut(v.xm[k], sigma);
-    x.yp[k] = h37::cut(v.yp[k], sigma);
-    x.ym[k] = h37::cut(v.ym[k], sigma);
-  }
-#pragma unroll
-  for (int k = 0; k < NQ; ++k) {
-    x.pp[k] = h37::cut(v.pp[k], sigma);
-    x.mp[k] = h37::cut(v.mp[k], sigma);
-    x.pm[k] = h37::cut(v.pm[k], sigma);
-    x.mm[k] = h37::cut(v.mm[k], sigma);
-  }
-  f2 M2[NC];
-  orbit_moments<f2>(rule.o, x, M2);
-  float M[NC], L[NC], H[NC], inc[NC], s[NC], c[NC];
-  h37::round_parts<NC>(M2, M, L);
-  h37::to_basis_exact<NC>(M, L, H, m);
-  const bool ok = h37::moment_increments<float, NC>(H, inc, m);
-  h37::add_increments<NC>(M, L, inc);
-  h37::to_polynomial_exact<NC>(M, L, rule.map, s, c);
-  f2 b[NC];
-  h37::cut_polynomial<NC>(s, c, b, kOrbitPolynomialBits);
-  orbit_values<f2>(rule.o, b, x, false);
-  v.r = h37::weigh(x.r, rule.w.w0);
-#pragma unroll
-  for (int k = 0; k < NA; ++k) {
-    v.xp[k] = h37::weigh(x.xp[k], rule.w.pw[k]);
-    v.xm[k] = h37::weigh(x.xm[k], rule.w.pw[k]);
-    v.yp[k] = h37::weigh(x.yp[k], rule.w.pw[k]);
-    v.ym[k] = h37::weigh(x.ym[k], rule.w.pw[k]);
-  }
-#pragma unroll
-  for (int k = 0; k < NQ; ++k) {
-    v.pp[k] = h37::weigh(x.pp[k], rule.w.qw[k]);
-    v.mp[k] = h37::weigh(x.mp[k], rule.w.qw[k]);
-    v.pm[k] = h37::weigh(x.pm[k], rule.w.qw[k]);
-    v.mm[k] = h37::weigh(x.mm[k], rule.w.qw[k]);
-  }
+  orbit_values<double>(rule.o, M, v);
   return ok;
 }
 
@@ -932,24 +857,11 @@ void fill_map(double c2, int, HMap* k) {
                         n * n * n / 6.0, 0.25 * n * n * n * n, n * n * n * n / 6.0, n * n * n * n / 24.0};
   for (int i = 0; i < 13; ++i) k->v[i] = v[i];
 }
-void fill_map(double c2, int nc, HSplitMap* k) {
-  for (int t = 0; t < h37::kMapTerms; ++t) k->v[t] = h37::split_of(h37::map_term(t, nc, c2));
-}
 template <int NA, int NQ>
 bool fill_rule(const HLattice& L, int nc, OrbitRule<double, NA, NQ>* r) {
   fill_map(L.c * L.c, nc, &r->map);
-  return make_orbits(L, true, &r->o);
+  return make_orbits(L, &r->o);
 }
-template <int NA, int NQ>
-bool fill_rule(const HLattice& L, int nc, OrbitRule<float, NA, NQ>* r) {
-  fill_map(L.c * L.c, nc, &r->map);
-  if (!make_orbits(L, false, &r->o)) return false;
-  r->w.w0 = h37::split_of(L.w[r->o.rest]);
-  for (int k = 0; k < NA; ++k) r->w.pw[k] = h37::split_of(L.w[r->o.xp[k]]);
-  for (int k = 0; k < NQ; ++k) r->w.qw[k] = h37::split_of(L.w[r->o.pp[k]]);
-  return true;
-}
-
 template <typename T>
 h37::MomentModel<T> hmoment_model(const Sim* s) {
   h37::MomentModel<T> m;
@@ -1015,7 +927,8 @@ cudaError_t sweep_e(Sim* s, int odd, const HSplit& sp) {
 // FP32 storage takes the correctly rounded transforms unless LBM_FAST_TRANSFORMS.
 template <int S, int Q, int NC>
 cudaError_t sweep_t(Sim* s, int odd) {
-  if (S == LBM_F64 || !(s->flags & LBM_FAST_TRANSFORMS)) {
+  // FP64 only: FP32 populations keep the roundings of the tables' collision
+  if constexpr (S == LBM_F64) {
     // the orbit counts of the minimal rules: 37 velocities have three axis shells, 17 one or two
     bool taken = false;
     cudaError_t e;

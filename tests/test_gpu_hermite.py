@@ -192,26 +192,22 @@ def test_two_threads_per_node_match_one(lbm, name, flags):
 
 
 @pytest.mark.parametrize("name", ["E7-A", "E7-D", "E9-A", "E9-C"])
-@pytest.mark.parametrize("storage", ["f64", "f32"])
 @pytest.mark.parametrize("dims", [(3, 3), (13, 7), (37, 263)])
-def test_orbit_sweep_matches_the_dense_tables(lbm, name, storage, dims):
+def test_orbit_sweep_matches_the_dense_tables(lbm, name, dims):
     """The sweep by reflection orbits against the dense tables, which take a rule
     whose weights differ within an orbit: the same rule with the weight of one
     velocity an ulp larger and of its opposite an ulp smaller (other orders of
-    summation in FP64; in FP32 both paths compute every moment and population to
-    below 2^-24 of the largest and round once, and relax from rounded moments,
-    which differ by a few roundings of the largest moment, ~0.03)."""
+    summation)."""
     e, w, c, n = gen_rules.rule(name)
     k = 1
     opp = next(i for i, v in enumerate(e) if tuple(v) == tuple(-e[k]))
     wb = w.copy()
     wb[k], wb[opp] = np.nextafter(w[k], 1.0), np.nextafter(w[k], 0.0)
     rho, u, theta = _fields(dims, seed=21)
-    sims = [lbm.HermiteSimulation((e, x, c, n), dims, TAUS, storage=storage, flags=lbm.LBM_THERMAL, theta_ref=1.1)
+    sims = [lbm.HermiteSimulation((e, x, c, n), dims, TAUS, storage="f64", flags=lbm.LBM_THERMAL, theta_ref=1.1)
             for x in (w, wb)]
     for s in sims:
         s.init_fields(rho, u, theta)
         s.step(5)
     a, b = (s.populations() for s in sims)
-    tol = 5e-14 if storage == "f64" else 5 * 16 * 2.0 ** -24 * 0.03
-    np.testing.assert_allclose(a, b, rtol=0, atol=tol)
+    np.testing.assert_allclose(a, b, rtol=0, atol=5e-14)
