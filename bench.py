@@ -790,11 +790,11 @@ def run_batch(args):
 
 
 THERMAL_N, THERMAL_THETA0, THERMAL_PR = 1024, 1.2, 0.71
-# FP32 arithmetic of one 37-velocity thermal lattice update, the one-node kernel's executed
-# counts (ncu, both parities): FP32 storage through the Hermite tables 2 x 515 FFMA + 172
-# FADD + 36 FMUL; 16-bit storage through raw moments 2 x 211 FFMA + 188 FADD + 75 FMUL
-# (FP64 storage takes the same steps).
-H37_FLOPS_PER_LUP = {8: 685.0, 4: 1238.0, 2: 685.0}  # by element size
+# FP32 arithmetic of one 37-velocity thermal lattice update through the Hermite tables:
+# 2 x 515 FFMA + 172 FADD + 36 FMUL, the one-node kernel's executed counts (ncu, both
+# parities); 16-bit offsets add 37 + 37 FMUL for the w_i scaling.  (FP64 storage, through
+# raw moments: 2 x 211 FFMA + 188 FADD + 75 FMUL.)
+H37_FLOPS_PER_LUP = {8: 685.0, 4: 1238.0, 2: 1238.0 + 74.0}  # by element size
 # FP32 ALU peak from unit counts: 128 FP32 FMA lanes per SM x 2 flop x SMs x SM clock.
 FP32_LANES_PER_SM = 128
 

@@ -39,7 +39,7 @@ h37::MomentModel<R> moment_model(const Sim* s) {
   h37::MomentModel<R> m;
   for (int n = 0; n < 5; ++n) m.no[n] = (R)-s->rates.w[n];
   m.s = (R)h37::kS;
-  const double tau = s->storage == LBM_F32 || s->storage == LBM_F64 ? h37::basis_temperature(s->theta_ref * h37::kS) : 0.0;
+  const double tau = h37::basis_temperature(s->theta_ref * h37::kS);
   m.basis = (R)tau;
   m.basis2x3 = (R)(3.0 * tau * tau);
   m.th_ref = (R)(s->theta_ref * h37::kS - tau);
@@ -48,49 +48,29 @@ h37::MomentModel<R> moment_model(const Sim* s) {
   m.usq_max = (R)(4.0 * h37::kS);
   m.thermal = b.thermal;
   m.raw = b.raw;
-  m.sround = b.sround;
-  m.seed = b.seed;
   return m;
 }
 
-// What a sweep takes and how it updates a node (or pair), by storage type.  Plain
-// FP32 transforms (FP32 storage with LBM_FAST_TRANSFORMS) stay on the Hermite
-// tables: their errors recur every step, and the row sums in FP32 drift twice as
-// fast (2.0e-5 against 1.1e-5 relative on the velocity after 1000 steps).
+// What a sweep takes, by storage type.  What is computed in plain FP32 (16-bit
+// storage, and FP32 with LBM_FAST_TRANSFORMS) takes the Hermite tables: errors of
+// the transforms recur every step, and row sums in plain FP32 drift twice as fast
+// (FP32 storage: 2.0e-5 against 1.1e-5 relative on the velocity after 1000 steps).
 struct TableModel {
   Rates r;
   h37::Model m;
 };
 template <int S, bool EXACT>
-using SweepModel = typename std::conditional<S == LBM_F32 && !EXACT, TableModel,
-                                             h37::MomentModel<typename h37::Store<S>::calc>>::type;
+constexpr bool kTables = S != LBM_F64 && !EXACT;
+template <int S, bool EXACT>
+using SweepModel =
+    typename std::conditional<kTables<S, EXACT>, TableModel, h37::MomentModel<typename h37::Store<S>::calc>>::type;
 template <int S, bool EXACT>
 SweepModel<S, EXACT> sweep_model(const Sim* s) {
-  if constexpr (S == LBM_F32 && !EXACT)
+  if constexpr (kTables<S, EXACT>)
     return TableModel{s->rates, model_of(s)};
   else
     return moment_model<typename h37::Store<S>::calc>(s);
 }
-// mom, if not null: drho and the momentum in lattice units
-template <typename T, bool SCALED>
-__device__ __forceinline__ bool update_values(T (&v)[h37::kQ], const TableModel& t, T* mom) {
-  T om[5];
-#pragma unroll
-  for (int n = 0; n < 5; ++n) om[n] = cst<T>(t.r.w[n]);
-  const bool ok = h37::collide<T>(v, om, t.m, mom);
-  if (mom) {
-    mom[1] = mom[1] * cst<T>(1.0 / h37::kC);
-    mom[2] = mom[2] * cst<T>(1.0 / h37::kC);
-  }
-  return ok;
-}
-template <typename T, bool SCALED, typename R>
-__device__ __forceinline__ bool update_values(T (&v)[h37::kQ], const h37::MomentModel<R>& m, T* mom) {
-  return h37::collide_rows<T, SCALED, !SCALED>(v, m, mom);
-}
-template <typename R>
-__device__ __forceinline__ const h37::MomentModel<R>& rounding(const h37::MomentModel<R>& m) { return m; }
-__device__ __forceinline__ const h37::Model& rounding(const TableModel& t) { return t.m; }
 
 inline h37::Grid2 grid2(const Sim* s) { return h37::Grid2{(int)s->nx, (int)s->ny, s->N}; }
 
@@ -107,70 +87,52 @@ inline bool h37_scalar_only() {
   return e && std::strcmp(e, "scalar") == 0;
 }
 
-// Stored value to the number the node update takes, and back (the update works on
-// f / w where that is what is stored).
-template <int S>
-__device__ __forceinline__ typename h37::Store<S>::calc unstore(typename h37::Store<S>::type s) {
-  if constexpr (S == LBM_F16)
-    return __half2float(s);
-  else if constexpr (S == LBM_BF16)
-    return __bfloat162float(s);
-  else
-    return s;
-}
-template <int S>
-__device__ __forceinline__ typename h37::Store<S>::type restore(typename h37::Store<S>::calc v) {
-  if constexpr (S == LBM_F16)
-    return __float2half_rn(v);
-  else if constexpr (S == LBM_BF16)
-    return __float2bfloat16_rn(v);
-  else
-    return v;
-}
-template <int S>
-__device__ __forceinline__ typename h37::Store<S>::type restore_sr(typename h37::Store<S>::calc v, uint32_t r) {
-  if constexpr (S == LBM_F16)
-    return __float2half_rz(h37::dither(v, r, 13));
-  else if constexpr (S == LBM_BF16)
-    return __float2bfloat16_rz(h37::dither(v, r, 16));
-  else
-    return v;
-}
-
 // EXACT: correctly rounded transforms (FP32 storage unless LBM_FAST_TRANSFORMS).
 // Threads walk the nodes of the grid in one dimension, so that rows of any
-// length fill the warps.
+// length fill the warps.  On the tables they are launched by rows and the stores keep
+// the loads' addresses: which products and sums the compiler merges there follows the
+// code around the collision, and the results are to keep their bits
+// (tests/test_gpu_h37_bits.py).
 template <int S, bool ODD, bool EXACT>
 __global__ void __launch_bounds__(kH37Threads)
     h37_sweep_kernel(typename h37::Store<S>::type* __restrict__ f, h37::Grid2 g,
                      SweepModel<S, EXACT> m, int* __restrict__ status) {
   using T = typename h37::Store<S>::calc;
-  constexpr bool kScaled = S == LBM_F16 || S == LBM_BF16;
-  const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
+  int x = (int)(blockIdx.x * blockDim.x + threadIdx.x), y = blockIdx.y;
   chain_wait();
-  if (node >= (uint32_t)g.N) return;
-  int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
+  if (kTables<S, EXACT> ? x >= g.nx : (uint32_t)x >= (uint32_t)g.N) return;
+  if constexpr (!kTables<S, EXACT>) {
+    const uint32_t node = (uint32_t)x;
+    y = (int)(node / (uint32_t)g.nx);
+    x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
+  }
   T v[h37::kQ];
-#pragma unroll
-  for (int j = 0; j < h37::kQ; ++j)
-    v[ODD ? h37::opp(j) : j] = unstore<S>(f[(size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : node)]);
+  h37::gather<S>(f, g, x, y, ODD ? 1 : 0, v);
   bool ok;
-  if constexpr (EXACT)
+  if constexpr (kTables<S, EXACT>) {
+    T om[5];
+#pragma unroll
+    for (int n = 0; n < 5; ++n) om[n] = (T)m.r.w[n];
+    ok = h37::collide<T>(v, om, m.m);
+  } else if constexpr (EXACT) {
     ok = h37::collide_exact(v, m);
-  else
-    ok = update_values<T, kScaled>(v, m, static_cast<T*>(nullptr));
+  } else {
+    ok = h37::collide_rows(v, m);
+  }
   if (!ok) atomicOr(status, 1);
   // even sweep: population i goes to slot (x, opp(i)); odd sweep: to slot (x + e_i, i)
-  // 16-bit storage: the stores' addresses anew, for twice the warps (the correctly
-  // rounded FP32 update is better off with them kept: 128^2 4.0 us a step, 4.6 so)
-  if constexpr (kScaled) forget(x, y);
   const uint32_t own = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
-  h37::SrStream rs(rounding(m).seed, own);
+  auto slot = [&](int j) { return (size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : own); };
+  if constexpr (kTables<S, EXACT>) {
+    h37::SrStream rs(m.m.seed, own);
 #pragma unroll
-  for (int j = 0; j < h37::kQ; ++j) {
-    const T val = ODD ? v[j] : v[h37::opp(j)];
-    const auto e = kScaled && rounding(m).sround ? restore_sr<S>(val, rs.next()) : restore<S>(val);
-    f[(size_t)j * g.N + (ODD ? h37::nbr(g, x, y, j) : own)] = e;
+    for (int j = 0; j < h37::kQ; ++j) {
+      const T val = ODD ? v[j] : v[h37::opp(j)];
+      f[slot(j)] = m.m.sround ? h37::encode_sr<S>(val, j, rs.next()) : h37::encode<S>(val, j);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < h37::kQ; ++j) f[slot(j)] = ODD ? v[j] : v[h37::opp(j)];
   }
 }
 
@@ -183,17 +145,17 @@ __global__ void __launch_bounds__(kH37Threads)
 // even e_x.
 //
 // 4 blocks per SM: with the stores' addresses computed anew instead of kept from the
-// loads the kernel takes 112 registers (168 before, at 3 blocks: FP16 1024^2 29.5
-// us a step, 27.7 so).
+// loads the kernel takes 112 to 128 registers (168 before, at 3 blocks).  FP16 1024^2,
+// us a step: 38.2 in plain launches, 35.3 chained at 3 blocks, 33.7 so.
 #ifndef LBM_H37_PAIR_MINB
 #define LBM_H37_PAIR_MINB 4
 #endif
 // The update of pair xp of row blockIdx.y; with TOT the pair's conserved
-// moments (drho, j_x, j_y, both lanes) go to mom[0..2].
+// moments (drho, j_x, j_y in Hermite units, both lanes) go to mom[0..2].
 template <int S, bool ODD, bool TOT>
 __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restrict__ f, const h37::Grid2& g,
-                                                const SweepModel<S, false>& m, int* __restrict__ status, int xp,
-                                                f2* mom) {
+                                                const TableModel& t, int* __restrict__ status, int xp, f2* mom) {
+  const h37::Model& m = t.m;
   using IO = PairIO<S>;
   using E = typename IO::E;
   int y = blockIdx.y;
@@ -205,6 +167,9 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
     yy = yy < 0 ? yy + g.ny : (yy >= g.ny ? yy - g.ny : yy);
     return (uint32_t)nx * (uint32_t)yy;
   };
+  f2 om[5];
+#pragma unroll
+  for (int n = 0; n < 5; ++n) om[n] = cst<f2>(t.r.w[n]);
   f2 v[h37::kQ];
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j) {
@@ -220,18 +185,20 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
       else
         val = IO::load11(fj + ro + wrapx(x0 + ex), fj + ro + wrapx(x0 + 1 + ex));
     }
+    if (IO::kScaled) val = val * cst<f2>(h37::w_of(j));
     v[ODD ? h37::opp(j) : j] = val;
   }
-  const bool ok = update_values<f2, IO::kScaled>(v, m, TOT ? mom : nullptr);
+  const bool ok = h37::collide<f2>(v, om, m, TOT ? mom : nullptr);
   if (!ok) atomicOr(status, 1);
   forget(x0, y);
   // the pair's own nodes (for the stochastic-rounding bits)
   const uint32_t n0 = (uint32_t)x0 + (uint32_t)nx * (uint32_t)y, n1 = (uint32_t)wrapx(x0 + 1) + (uint32_t)nx * (uint32_t)y;
-  h37::SrStream rs0(rounding(m).seed, n0), rs1(rounding(m).seed, n1);
+  h37::SrStream rs0(m.seed, n0), rs1(m.seed, n1);
 #pragma unroll
   for (int j = 0; j < h37::kQ; ++j) {
     E* fj = f + (size_t)j * g.N;
     f2 val = ODD ? v[j] : v[h37::opp(j)];
+    if (IO::kScaled) val = val * cst<f2>(1.0 / h37::w_of(j));
     E* pa;
     E* pb;
     bool adjacent;
@@ -247,7 +214,7 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
       adjacent = (ex & 1) != 0;
     }
     if constexpr (S == LBM_F16 || S == LBM_BF16) {
-      if (rounding(m).sround) {
+      if (m.sround) {
         float lo, hi;
         unpack2(val, lo, hi);
         const uint32_t r0 = rs0.next(), r1 = rs1.next();
@@ -270,7 +237,7 @@ __device__ __forceinline__ void h37_pair_update(typename PairIO<S>::E* __restric
 
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
-    h37_pair_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, SweepModel<S, false> m,
+    h37_pair_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, TableModel m,
                     int* __restrict__ status) {
   const int xp = blockIdx.x * blockDim.x + threadIdx.x;
   chain_wait();
@@ -284,7 +251,7 @@ __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
 // partials[warp * 8 + k]; a warp sums its 64 nodes in FP32 (fixed shuffle tree).
 template <int S, bool ODD>
 __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
-    h37_pair_totals_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, SweepModel<S, false> m,
+    h37_pair_totals_kernel(typename PairIO<S>::E* __restrict__ f, h37::Grid2 g, TableModel m,
                            int* __restrict__ status, float* __restrict__ partials) {
   const int xp = blockIdx.x * blockDim.x + threadIdx.x;
   float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
@@ -292,10 +259,15 @@ __global__ void __launch_bounds__(kH37Threads, LBM_H37_PAIR_MINB)
   if (2 * xp < g.nx) {
     f2 mom[3];
     h37_pair_update<S, ODD, true>(f, g, m, status, xp, mom);
+    const float ic = (float)(1.0 / h37::kC);
     float d0, d1, jx0, jx1, jy0, jy1;
     unpack2(mom[0], d0, d1);
     unpack2(mom[1], jx0, jx1);
     unpack2(mom[2], jy0, jy1);
+    jx0 *= ic;
+    jx1 *= ic;
+    jy0 *= ic;
+    jy1 *= ic;
     acc[0] = d0 + d1;
     acc[1] = jx0 + jx1;
     acc[2] = jy0 + jy1;
@@ -509,11 +481,13 @@ cudaError_t sweep_t(Sim* s, int odd) {
     if (h37_pair_supported(s)) return pair_t<S>(s, odd);
   }
   const int t = node_threads(s->N);
-  const unsigned blocks = (unsigned)((s->N + t - 1) / t);
   E* f = static_cast<E*>(s->pop);
   auto launch = [&](auto odd_c, auto exact_c) {
-    return launch_chained(h37_sweep_kernel<S, decltype(odd_c)::value, decltype(exact_c)::value>, dim3(blocks), dim3(t), 0,
-                          s->stream, f, grid2(s), sweep_model<S, decltype(exact_c)::value>(s), status_word(s));
+    constexpr bool odd_v = decltype(odd_c)::value, exact_v = decltype(exact_c)::value;
+    const dim3 blocks = kTables<S, exact_v> ? dim3((unsigned)((s->nx + t - 1) / t), (unsigned)s->ny)
+                                            : dim3((unsigned)((s->N + t - 1) / t));
+    return launch_chained(h37_sweep_kernel<S, odd_v, exact_v>, blocks, dim3(t), 0, s->stream, f, grid2(s),
+                          sweep_model<S, exact_v>(s), status_word(s));
   };
   if constexpr (S == LBM_F32) {
     if (h37_exact_transforms(s))

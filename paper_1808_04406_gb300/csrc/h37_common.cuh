@@ -402,6 +402,18 @@ __device__ __forceinline__ typename Store<S>::calc decode(typename Store<S>::typ
     return __bfloat162float(s) * (float)w_of(i);
   }
 }
+// Stochastically rounded encode (FP16 / BF16; the other types round as encode).
+template <int S>
+__device__ __forceinline__ typename Store<S>::type encode_sr(typename Store<S>::calc v, int i, uint32_t r) {
+  if constexpr (S == LBM_F64 || S == LBM_F32) {
+    return v;
+  } else if constexpr (S == LBM_F16) {
+    return __float2half_rz(dither(v * (float)(1.0 / w_of(i)), r, 13));
+  } else {
+    return __float2bfloat16_rz(dither(v * (float)(1.0 / w_of(i)), r, 16));
+  }
+}
+
 template <int S>
 __device__ __forceinline__ typename Store<S>::type encode(typename Store<S>::calc v, int i) {
   if constexpr (S == LBM_F64 || S == LBM_F32) {

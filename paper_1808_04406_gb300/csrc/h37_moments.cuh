@@ -13,13 +13,11 @@
 // +- pairs folded).  Arithmetic and instruction fetch bound these kernels (all of
 // an update is straight-line code, 96 KB of it for the FP32 sweep with
 // compensated table sums, whose warps waited for instructions 78 % of the time).
-// Microseconds a step, before and after: thermal FP16 1024^2 38.2 and 31.9, FP32
-// (correctly rounded) 512^2 66.5 and 20.3, 128^2 14.3 and 6.1 (27.6, 18.2 and 4.0 since
-// the steps are chained launches and the pair sweep runs at 4 blocks per SM).
+// Microseconds a step, before and after, FP32 (correctly rounded): 512^2 66.5 and
+// 20.3, 128^2 14.3 and 6.1 (18.2 and 4.0 since the steps are chained launches).
 //
-// 16-bit storage holds f_i / w_i: the weights then go into the row constants on
-// the way in (no extra operation for a row, five for the middle one), and P(e_i)
-// is stored as it is.
+// FP64, and FP32 with error-free sums, only: plain FP32 sums of raw moments drift
+// twice as fast as the tables' (h37.cu).
 #pragma once
 
 #include <cmath>
@@ -48,43 +46,38 @@ __device__ __forceinline__ T axpy(double k, T x, T m) {
   return k == 1.0 ? m + x : fma_(x, cst<T>(k), m);
 }
 
-// x moments 0..4 of row EY: of f, or with SCALED of f / w(1, EY) from the stored f / w
-template <typename T, bool SCALED, int EY>
+// x moments 0..4 of row EY
+template <typename T, int EY>
 __device__ __forceinline__ void row_moments(const T (&v)[kQ], T (&r)[5]) {
   constexpr int H = row_half(EY);
-  constexpr double w1 = w_at(1, EY);
-  constexpr double r0 = SCALED ? w_at(0, EY) / w1 : 1.0;
   const T s1 = v[vidx(1, EY)] + v[vidx(-1, EY)], d1 = v[vidx(1, EY)] - v[vidx(-1, EY)];
-  r[0] = axpy(r0, v[vidx(0, EY)], s1);
+  r[0] = s1 + v[vidx(0, EY)];
   r[1] = r[3] = d1;
   r[2] = r[4] = s1;
   if constexpr (H >= 2) {
-    constexpr double r2 = SCALED ? w_at(2, EY) / w1 : 1.0;
     const T s2 = v[vidx(2, EY)] + v[vidx(-2, EY)], d2 = v[vidx(2, EY)] - v[vidx(-2, EY)];
-    r[0] = axpy(r2, s2, r[0]);
-    r[1] = axpy(2.0 * r2, d2, r[1]);
-    r[2] = axpy(4.0 * r2, s2, r[2]);
-    r[3] = axpy(8.0 * r2, d2, r[3]);
-    r[4] = axpy(16.0 * r2, s2, r[4]);
+    r[0] = r[0] + s2;
+    r[1] = axpy(2.0, d2, r[1]);
+    r[2] = axpy(4.0, s2, r[2]);
+    r[3] = axpy(8.0, d2, r[3]);
+    r[4] = axpy(16.0, s2, r[4]);
   }
   if constexpr (H >= 3) {
-    constexpr double r3 = SCALED ? w_at(3, EY) / w1 : 1.0;
     const T s3 = v[vidx(3, EY)] + v[vidx(-3, EY)], d3 = v[vidx(3, EY)] - v[vidx(-3, EY)];
-    r[0] = axpy(r3, s3, r[0]);
-    r[1] = axpy(3.0 * r3, d3, r[1]);
-    r[2] = axpy(9.0 * r3, s3, r[2]);
-    r[3] = axpy(27.0 * r3, d3, r[3]);
-    r[4] = axpy(81.0 * r3, s3, r[4]);
+    r[0] = r[0] + s3;
+    r[1] = axpy(3.0, d3, r[1]);
+    r[2] = axpy(9.0, s3, r[2]);
+    r[3] = axpy(27.0, d3, r[3]);
+    r[4] = axpy(81.0, s3, r[4]);
   }
 }
 
 // add rows +B and -B to the moments
-template <typename T, bool SCALED, int B>
+template <typename T, int B>
 __device__ __forceinline__ void add_rows(const T (&v)[kQ], T (&M)[kNC]) {
-  constexpr double w = SCALED ? w_at(1, B) : 1.0;
   T a[5], b[5];
-  row_moments<T, SCALED, B>(v, a);
-  row_moments<T, SCALED, -B>(v, b);
+  row_moments<T, B>(v, a);
+  row_moments<T, -B>(v, b);
   constexpr bool narrow = row_half(B) == 1;  // then r2 = r4 and r1 = r3
   T e[5], o[4];
 #pragma unroll
@@ -92,44 +85,40 @@ __device__ __forceinline__ void add_rows(const T (&v)[kQ], T (&M)[kNC]) {
 #pragma unroll
   for (int p = 0; p < 4; ++p) o[p] = narrow && p > 2 ? o[p - 2] : a[p] - b[p];
 #pragma unroll
-  for (int p = 0; p < 5; ++p) M[cidx(p, 0)] = axpy(w, e[p], M[cidx(p, 0)]);
+  for (int p = 0; p < 5; ++p) M[cidx(p, 0)] = M[cidx(p, 0)] + e[p];
 #pragma unroll
-  for (int p = 0; p < 4; ++p) M[cidx(p, 1)] = axpy(w * B, o[p], M[cidx(p, 1)]);
+  for (int p = 0; p < 4; ++p) M[cidx(p, 1)] = axpy(B, o[p], M[cidx(p, 1)]);
 #pragma unroll
-  for (int p = 0; p < 3; ++p) M[cidx(p, 2)] = axpy(w * B * B, e[p], M[cidx(p, 2)]);
+  for (int p = 0; p < 3; ++p) M[cidx(p, 2)] = axpy(B * B, e[p], M[cidx(p, 2)]);
 #pragma unroll
-  for (int p = 0; p < 2; ++p) M[cidx(p, 3)] = axpy(w * B * B * B, o[p], M[cidx(p, 3)]);
-  M[cidx(0, 4)] = axpy(w * B * B * B * B, e[0], M[cidx(0, 4)]);
+  for (int p = 0; p < 2; ++p) M[cidx(p, 3)] = axpy(B * B * B, o[p], M[cidx(p, 3)]);
+  M[cidx(0, 4)] = axpy(B * B * B * B, e[0], M[cidx(0, 4)]);
 }
 
 // rows +1 and -1 start the sums over e_y != 0 (so that no addition to zero is left)
-template <typename T, bool SCALED>
+template <typename T>
 __device__ __forceinline__ void to_moments(const T (&v)[kQ], T (&M)[kNC]) {
-  constexpr double w0 = SCALED ? w_at(1, 0) : 1.0;
   T r[5];
-  row_moments<T, SCALED, 0>(v, r);
+  row_moments<T, 0>(v, r);
 #pragma unroll
-  for (int p = 0; p < 5; ++p) M[cidx(p, 0)] = SCALED ? r[p] * cst<T>(w0) : r[p];
-  constexpr double w = SCALED ? w_at(1, 1) : 1.0;
+  for (int p = 0; p < 5; ++p) M[cidx(p, 0)] = r[p];
   T a[5], b[5];
-  row_moments<T, SCALED, 1>(v, a);
-  row_moments<T, SCALED, -1>(v, b);
+  row_moments<T, 1>(v, a);
+  row_moments<T, -1>(v, b);
 #pragma unroll
   for (int p = 0; p < 5; ++p) {
     const T e = a[p] + b[p];
-    M[cidx(p, 0)] = axpy(w, e, M[cidx(p, 0)]);
-    const T we = SCALED && p < 3 ? e * cst<T>(w) : e;
-    if (p < 3) M[cidx(p, 2)] = we;
-    if (p == 0) M[cidx(0, 4)] = we;
+    M[cidx(p, 0)] = M[cidx(p, 0)] + e;
+    if (p < 3) M[cidx(p, 2)] = e;
+    if (p == 0) M[cidx(0, 4)] = e;
     if (p < 4) {
       const T o = a[p] - b[p];
-      const T wo = SCALED ? o * cst<T>(w) : o;
-      M[cidx(p, 1)] = wo;
-      if (p < 2) M[cidx(p, 3)] = wo;
+      M[cidx(p, 1)] = o;
+      if (p < 2) M[cidx(p, 3)] = o;
     }
   }
-  add_rows<T, SCALED, 2>(v, M);
-  add_rows<T, SCALED, 3>(v, M);
+  add_rows<T, 2>(v, M);
+  add_rows<T, 3>(v, M);
 }
 
 // Row EY and -EY of the populations from the polynomial's coefficients.
@@ -253,7 +242,7 @@ template <typename R>
 struct MomentModel {
   R no[5];      // minus the rates of orders 2..4
   R s;          // 1 / c^2
-  R basis;      // temperature tau of the Hermite basis the collision takes its moments in (0: plain moments)
+  R basis;      // temperature tau of the Hermite basis the collision takes its moments in
   R basis2x3;   // 3 tau^2
   R th_ref;     // theta_ref / c^2 - tau
   R th_iso;     // temperature of isothermal runs, 1 / c^2 - tau
@@ -261,8 +250,6 @@ struct MomentModel {
   R usq_max;    // the largest |u|^2 the collision is defined on
   int thermal;
   int raw;      // relax in the absolute frame (the shifts to and from the relative frame are left out)
-  int sround;   // stochastic rounding of FP16 / BF16 stores
-  uint32_t seed;
 };
 
 template <typename T>
@@ -731,7 +718,7 @@ __device__ __forceinline__ bool collide_exact(float (&v)[kQ], const MomentModel<
     f2 x[kQ], M2[kNC];
 #pragma unroll
     for (int i = 0; i < kQ; ++i) x[i] = cut(v[i], sigma);
-    to_moments<f2, false>(x, M2);
+    to_moments(x, M2);
     round_parts<kNC>(M2, M, L);
   }
   float H[kNC];
@@ -747,33 +734,16 @@ __device__ __forceinline__ bool collide_exact(float (&v)[kQ], const MomentModel<
   return ok;
 }
 
-// One node (or node pair) of the built-in rule.  v: offsets, divided by the
-// weights with SCALED, in and out.  mom, if not null, receives drho and the
-// momentum (lattice units), which the collision leaves unchanged.
-// BASIS: collide in the reference's Hermite basis (m.basis is then its temperature, else 0).
-template <typename T, bool SCALED, bool BASIS>
-__device__ __forceinline__ bool collide_rows(T (&v)[kQ], const MomentModel<typename real_of<T>::type>& m,
-                                             T* mom = nullptr) {
-  T M[kNC];
-  to_moments<T, SCALED>(v, M);
-  if (mom) {
-    mom[0] = M[0];
-    mom[1] = M[cidx(1, 0)];
-    mom[2] = M[cidx(0, 1)];
-  }
-  T inc[kNC];
-  bool ok;
-  if constexpr (BASIS) {
-    T H[kNC];
-    to_basis<T, kNC>(M, H, m);
-    ok = moment_increments<T, kNC>(H, inc, m);
-  } else {
-    ok = moment_increments<T, kNC>(M, inc, m);
-  }
+// One node of the built-in rule, in FP64.  v: offsets, in and out.
+__device__ __forceinline__ bool collide_rows(double (&v)[kQ], const MomentModel<double>& m) {
+  double M[kNC], H[kNC], inc[kNC];
+  to_moments(v, M);
+  to_basis<double, kNC>(M, H, m);
+  const bool ok = moment_increments<double, kNC>(H, inc, m);
 #pragma unroll
   for (int k = 3; k < kNC; ++k) M[k] = M[k] + inc[k];
-  to_polynomial<T, kNC>(M, BuiltInMap<T>());
-  from_polynomial<T, SCALED>(M, v);
+  to_polynomial<double, kNC>(M, BuiltInMap<double>());
+  from_polynomial<double, false>(M, v);
   return ok;
 }
 

@@ -876,8 +876,6 @@ h37::MomentModel<T> hmoment_model(const Sim* s) {
   m.usq_max = (T)(4.0 * sl);
   m.thermal = (s->flags & LBM_THERMAL) ? 1 : 0;
   m.raw = 0;
-  m.sround = 0;
-  m.seed = 0;
   return m;
 }
 
