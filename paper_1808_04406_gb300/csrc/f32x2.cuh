@@ -44,6 +44,17 @@ __device__ __forceinline__ f2 fma_(f2 a, f2 b, f2 c) {
   return d;
 }
 
+// A product that the compiler must not merge into an FMA.  (A packed product and sum
+// are merged even when both say .rn: its lanes are multiplied one by one.)
+__device__ __forceinline__ float mul_apart(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_apart(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ f2 mul_apart(f2 a, f2 b) {
+  float a0, a1, b0, b1;
+  unpack2(a, a0, a1);
+  unpack2(b, b0, b1);
+  return pack2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+
 // ---- the same vocabulary for scalar compute types -----------------------------
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }

@@ -524,29 +524,19 @@ struct BuiltInSplitMap {
   __device__ __forceinline__ Split at(int t) const { return split_of(map_term(t, kNC, kC * kC)); }
 };
 
-// A product that the compiler must not merge into an FMA: the error terms below
-// are those of the rounded product.  (A packed product and sum are merged even
-// when both say .rn: its lanes are multiplied one by one.)
-__device__ __forceinline__ float prod_(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ f2 prod_(f2 a, f2 b) {
-  float a0, a1, b0, b1;
-  unpack2(a, a0, a1);
-  unpack2(b, b0, b1);
-  return pack2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
-}
-
-// s + c = sum of products of (x + xl) and h, s the rounded sum and c its error to second order
+// s + c = sum of products of (x + xl) and h, s the rounded sum and c its error to second
+// order (the error terms are those of the rounded products)
 template <typename T>
 struct Dot2 {
   T s, c;
   __device__ __forceinline__ Dot2(T x, T xl, Split h) {
     const T hh = spread<T>(h.h);
-    s = prod_(x, hh);
+    s = mul_apart(x, hh);
     c = fma_(xl, hh, fma_(x, spread<T>(h.l), fma_(x, hh, neg_(s))));
   }
   __device__ __forceinline__ void add(T x, T xl, Split h) {
     const T hh = spread<T>(h.h);
-    const T p = prod_(x, hh);
+    const T p = mul_apart(x, hh);
     const T t = s + p;
     const T z = t - s;
     const T e = (s - (t - z)) + (p - z);
@@ -660,7 +650,7 @@ __device__ __forceinline__ void to_basis_exact(const float (&M)[NC], const float
                                                const MomentModel<float>& m) {
   const float t = m.basis, t3 = 3.f * t, t6 = 6.f * t;
   auto sub = [&](float& h, float& l, float k, int i) {  // h + l -= k (M_i + L_i), k of at most 24 bits
-    const float p = prod_(k, M[i]), d = h - p;
+    const float p = mul_apart(k, M[i]), d = h - p;
     l += (two_sum_err(h, -p, d) - __fmaf_rn(k, M[i], -p)) - k * L[i];
     h = d;
   };

@@ -7,6 +7,8 @@
 // Population storage holds offsets from the rest equilibrium w_i.
 #pragma once
 
+#include <type_traits>
+
 #include "f32x2.cuh"
 #include "lbm_internal.cuh"
 
@@ -232,7 +234,10 @@ struct NodeMoments {
   T drho, j[D];
 };
 
-template <typename T, int D, bool MOM = false>
+//
+// APART: u^2 is a product by itself, as in the scalar types.  The packed sweeps on
+// D2Q9 leave it to the compiler, which merges it into u_x^2 + u_y^2.
+template <typename T, int D, bool MOM = false, bool APART = !std::is_same<T, f2>::value>
 __device__ __forceinline__ bool collide(T (&v)[qof<D>()], const T (&om)[2 * D + 1],
                                         NodeMoments<T, D>* mom = nullptr) {
   pops_to_raw<T, D>(v);
@@ -249,7 +254,7 @@ __device__ __forceinline__ bool collide(T (&v)[qof<D>()], const T (&om)[2 * D + 
   for (int d = 0; d < D; ++d) {
     w.u[d] = v[p3(d)] * irho;
     w.nu[d] = neg_(w.u[d]);
-    w.usq[d] = w.u[d] * w.u[d];
+    w.usq[d] = APART ? mul_apart(w.u[d], w.u[d]) : w.u[d] * w.u[d];
     w.nusq[d] = neg_sq(w.nu[d], w.u[d], w.usq[d]);
     w.kk2[d] = w.usq[d] + cst<T>(1.0 / 3.0);
   }

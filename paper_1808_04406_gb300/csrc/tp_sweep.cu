@@ -49,7 +49,9 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_SWEEP_MINB)
 // each of two rows is read and written in 1-element accesses along x that
 // coalesce.  Half the instructions of one node per thread.  On the last row of an
 // odd ny, lane 1 repeats lane 0's node: both lanes load the same slots, compute
-// the same values and store them twice to the same places.
+// the same values and store them twice to the same places.  Populations are those of
+// one node per thread bit for bit (tests/test_gpu_odd_rows.py): which kernel a grid
+// takes, or a slab of its planes, does not show.
 // us a step with one node per thread and so: D3Q27 FP32 161 x 95 x 77 47.7 and 42.0,
 // 241 x 200 x 200 369 and 322, FP16 129 x 128 x 128 69.7 and 57.1; D2Q9 BF16 1023^2 9.9
 // and 9.3, but FP32 1023 x 1024 9.8 and 10.2.  Grids of less than a wave of blocks
@@ -115,7 +117,7 @@ __global__ void __launch_bounds__(kSweepThreads, D == 3 ? 4 : 6)
   }
   // the stores' addresses are computed anew: kept from the loads they would take too many registers
   forget(x, y, z);
-  if (!tp::collide<f2, D>(v, om)) atomicOr(status, 1);
+  if (!tp::collide<f2, D, false, D == 2>(v, om)) atomicOr(status, 1);
   const ColumnPair<D, ODD> A(g, x, y, z);
 #pragma unroll
   for (int j = 0; j < tp::qof<D>(); ++j) {
