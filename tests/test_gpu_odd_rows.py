@@ -3,7 +3,7 @@ thread; the populations do not depend on it, bit for bit."""
 import numpy as np
 import pytest
 
-from paper_1808_04406_gb300 import inputs
+from paper_1808_04406_gb300 import inputs, slab
 
 pytestmark = pytest.mark.gpu
 
@@ -45,3 +45,28 @@ def test_copies_of_a_small_grid_evolve_as_it_does(lbm, lattice, dims, copies, st
         many.step(n)
         assert torch.equal(_bits(one.raw_populations()).tile(1, copies), _bits(many.raw_populations()))
     assert one.status() == many.status() == lbm.LBM_OK
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("dims,world", [((97, 64, 31), 2), ((97, 64, 31), 3), ((99, 63, 26), 2)])
+def test_slabs_below_the_switch_equal_the_whole_grid_above_it(lbm, dims, world, storage):
+    """A grid of 608 blocks of column pairs or more, cut into slabs that have fewer and
+    so take one node per thread: the owned populations are the whole grid's."""
+    taus = [0.53, 1.0, 0.53, 1.0, 0.53]
+    rho, u = inputs.random_noise(dims, seed=23, du=0.05, drho=0.02)
+    whole = lbm.Simulation("D3Q27", dims, taus, storage=storage)
+    whole.init_fields(rho, u)
+    runs = [slab.SlabRun.create(dims, taus, storage, r, world) for r in range(world)]
+    assert whole.sweep_kernel() == "tp_column_kernel" and all(r.sim.sweep_kernel() == "tp_sweep_kernel" for r in runs)
+    for run in runs:
+        run.sim.init_fields(*run.local_fields(rho, u))
+    group = slab.LocalGroup(runs)
+    for n in (2, 5):
+        whole.step(n)
+        group.step(n)
+        group.refresh_ghosts()  # odd parity: boundary nodes read populations from the ghost planes
+        f = whole.populations().reshape(27, dims[2], -1)
+        for run in runs:
+            own = run.owned(run.sim.populations(), 27).reshape(27, run.nzl, -1)
+            np.testing.assert_array_equal(own, f[:, run.z0:run.z0 + run.nzl])
+    assert whole.status() == lbm.LBM_OK
