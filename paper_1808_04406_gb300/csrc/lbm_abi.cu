@@ -232,9 +232,11 @@ cudaError_t launch_reduce_into(Sim* s, double* partials, int nblocks, double* re
 
 // n steps, several per launch where that is possible
 static int advance(Sim* s, int64_t n) {
+  bool several = true;
   while (n > 0) {
     int done = 0;
-    cudaError_t e = launch_steps(s, n, &done);
+    cudaError_t e = several ? launch_steps(s, n, &done) : cudaSuccess;
+    several = done > 0;
     if (e == cudaSuccess && done < 1) {
       e = launch_sweep(s);
       done = 1;

@@ -23,6 +23,8 @@
 // fence, of which an SM does one at a time in ~0.3 us.
 #pragma once
 
+#include <cuda.h>
+
 #include "flat_index.cuh"
 #include "lbm_internal.cuh"
 
@@ -139,18 +141,30 @@ __global__ void __launch_bounds__(Up::kThreads, Up::kMinBlocks)
   }
 }
 
-// Resident blocks of a kernel on the current device (looked up once).
-template <typename Up>
-int multi_resident_blocks() {
-  static const int blocks = [] {
-    int dev = 0, sms = 0, per = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, multi_step_kernel<Up>, Up::kThreads, 0) != cudaSuccess)
-      return 0;
-    return sms * per;
+// Whether the stream's work may run on some of the device's SMs only.
+inline bool multi_green_context(cudaStream_t stream) {
+  using GetGreenCtx = CUresult (*)(CUstream, CUgreenCtx*);
+  static const GetGreenCtx get = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &p, 12040, cudaEnableDefault, &found);
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<GetGreenCtx>(p) : nullptr;
   }();
-  return blocks;
+  CUgreenCtx green = nullptr;
+  return get && get(stream, &green) == CUDA_SUCCESS && green != nullptr;
+}
+
+// Blocks of the kernel that are resident at once on the current device for work of this
+// stream, 0 if that is not known: in a green context, which has fewer SMs, a launch that
+// counts on all of them would be refused.
+template <typename Up>
+int multi_resident_blocks(cudaStream_t stream) {
+  int dev = 0, sms = 0, per = 0;
+  if (multi_green_context(stream) || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, multi_step_kernel<Up>, Up::kThreads, 0) != cudaSuccess)
+    return 0;
+  return sms * per;
 }
 
 // How much of the 129 MB L2 the populations between the first and the last step may

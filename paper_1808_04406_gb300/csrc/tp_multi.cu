@@ -59,12 +59,11 @@ cudaError_t run(Sim* s, int64_t n, int* done) {
   const int64_t plane_blocks = (s->ny * per_row + Up::kThreads - 1) / Up::kThreads;
   if (plane_blocks * Up::kThreads >= (int64_t)1 << 32) return cudaSuccess;
   const double bytes = (double)s->N * s->Q * (double)storage_elem_bytes(s->storage);
-  const int blocks = multi_resident_blocks<Up>();
+  const int blocks = multi_resident_blocks<Up>(s->stream);
   MultiPlan plan;
   // 2D: a node reaches the rows above and below, anywhere along them (periodic in x)
   multi_plan(n, s->D == 3 ? s->nz : 0, plane_blocks, 2.0 * per_row / Up::kThreads, bytes, blocks, (int)(s->step & 1),
              &plan);
-  *done = plan.steps;
   if (plan.steps < 2) return cudaSuccess;
   TpGrid p;
   p.g = tp::Grid{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
@@ -72,7 +71,13 @@ cudaError_t run(Sim* s, int64_t n, int* done) {
   p.f = s->pop;
   p.row = row_length(per_row);
   p.unit_blocks = plan.sub;
-  return multi_launch<Up>(s, p, plan, blocks);
+  const cudaError_t e = multi_launch<Up>(s, p, plan, blocks);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();  // not enough SMs for this stream: single sweeps need none
+    return cudaSuccess;
+  }
+  if (e == cudaSuccess) *done = plan.steps;
+  return e;
 }
 
 }  // namespace
