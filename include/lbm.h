@@ -270,6 +270,13 @@ int lbm_set_active_planes(lbm_handle h, int64_t z_lo, int64_t z_count);
  * same arithmetic.  Measurement and tests only; the string is static.  NULL for a NULL handle (no error code). */
 const char* lbm_sweep_kernel(lbm_handle h);
 
+/* Steps that the first launch of lbm_step(h, n) takes with the current settings
+ * (environment switches included): 1 where every step is a launch of its own, as on
+ * every grid but D2Q9 / D3Q27 ones with FP32 storage, even nx, no closure and
+ * more populations than L2 holds.  Measurement and tests only.  LBM_EINVAL for a
+ * NULL handle or n < 1. */
+int64_t lbm_steps_per_launch(lbm_handle h, int64_t n);
+
 /* Failure-detection self-test.  The paper has no counterpart; it exercises the
  * give-up path of the library's bounded device waits without a fault.  The
  * tensor-core sweeps wait on an mbarrier for their MMAs with a poll limit; a

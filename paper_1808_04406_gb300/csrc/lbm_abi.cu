@@ -21,7 +21,7 @@ const char* tp_pair_kernel_name(const Sim* s);
 // tp_sweep.cu: that of tp_launch_sweep.
 const char* tp_sweep_kernel_name(const Sim* s);
 // tp_multi.cu: up to n steps in one launch; *done = steps taken (0: one sweep at a time only).
-cudaError_t tp_launch_steps(Sim* s, int64_t n, int* done);
+cudaError_t tp_launch_steps(Sim* s, int64_t n, const StepsCall& call, int* done);
 
 static thread_local char g_err[512] = "";
 
@@ -216,12 +216,14 @@ cudaError_t launch_sweep(Sim* s) {
 }
 
 // up to n steps in one launch; *done = 0 where only single sweeps are possible
-cudaError_t launch_steps(Sim* s, int64_t n, int* done) {
+cudaError_t launch_steps(Sim* s, int64_t n, int* done, StepsCall call = StepsCall()) {
   *done = 0;
-  // LBM_MULTI_STEP=0 keeps one launch per step (read at every call; used to compare the two)
+  // LBM_MULTI_STEP=0 keeps one launch per step, LBM_MULTI_STEP=always puts several into one
+  // on grids of every size (read at every call; used to compare the two)
   const char* e = std::getenv("LBM_MULTI_STEP");
   if (n < 2 || s->closure || s->z_cnt > 0 || (e && std::strcmp(e, "0") == 0)) return cudaSuccess;
-  return hermite_family(s) ? cudaSuccess : tp_launch_steps(s, n, done);
+  call.any_size = e && std::strcmp(e, "always") == 0;
+  return hermite_family(s) ? cudaSuccess : tp_launch_steps(s, n, call, done);
 }
 
 cudaError_t launch_reduce_into(Sim* s, double* partials, int nblocks, double* result) {
@@ -759,6 +761,17 @@ const char* lbm_sweep_kernel(lbm_handle h) {
   if (is_h37(s)) return h37_pair_supported(s) ? "h37_pair_kernel" : "h37_sweep_kernel";
   if (s->closure) return closure_uses_tcgen05() ? "learned_tc_kernel" : "learned_sweep_kernel";
   return tp_pair_supported(s) ? tp_pair_kernel_name(s) : tp_sweep_kernel_name(s);
+}
+
+int64_t lbm_steps_per_launch(lbm_handle h, int64_t n) {
+  Sim* s = as_sim(h);
+  if (int rc = check_handle(s)) return rc;
+  if (n < 1) return set_error(LBM_EINVAL, "step count must be >= 1");
+  StepsCall count;
+  count.launch = false;
+  int done = 0;
+  if (int rc = cuda_check(launch_steps(s, n, &done, count), "plan of several steps")) return rc;
+  return done > 1 ? done : 1;
 }
 
 int lbm_selftest_wait_timeout(lbm_handle h, int polls) {

@@ -59,6 +59,12 @@ struct HTables {
   double c;
 };
 
+// How several steps are put into one launch (tp_multi.cu).
+struct StepsCall {
+  bool any_size = false;  // also on grids that stay in L2 by themselves (tests)
+  bool launch = true;     // else only count the steps
+};
+
 struct Sim {
   int lattice;
   int D, Q;

@@ -181,12 +181,12 @@ constexpr int kMultiMaxSub = 2;
 // Plan of up to n steps over `planes` planes of `plane_blocks` blocks of nodes (3D),
 // or over one run of plane_blocks blocks (planes = 0, 2D) whose velocities reach
 // `reach_blocks` blocks (rounded up) on either side; `bytes` of populations in all
-// and G resident blocks.  plan->steps < 2 where several steps at a time are not
-// possible.
+// and G resident blocks.  any_size: also where the whole grid stays in L2.
+// plan->steps < 2 where several steps at a time are not possible.
 inline void multi_plan(int64_t n, int64_t planes, int64_t plane_blocks, double reach_blocks, double bytes, int G,
-                       int first_odd, MultiPlan* plan) {
+                       int first_odd, bool any_size, MultiPlan* plan) {
   plan->steps = 0;
-  if (n < 2 || G < 1 || bytes <= (double)kResidentBytes) return;
+  if (n < 2 || G < 1 || (bytes <= (double)kResidentBytes && !any_size)) return;
   const int64_t blocks = (planes ? planes : 1) * plane_blocks;
   // two tiles or more per block and step, so that waits overlap with work
   int64_t sub = blocks / (2 * G);

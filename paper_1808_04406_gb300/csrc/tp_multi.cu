@@ -54,7 +54,7 @@ struct PairUp {
 };
 
 template <typename Up>
-cudaError_t run(Sim* s, int64_t n, int* done) {
+cudaError_t run(Sim* s, int64_t n, const StepsCall& call, int* done) {
   const int64_t per_row = s->nx / 2;
   const int64_t plane_blocks = (s->ny * per_row + Up::kThreads - 1) / Up::kThreads;
   if (plane_blocks * Up::kThreads >= (int64_t)1 << 32) return cudaSuccess;
@@ -63,8 +63,12 @@ cudaError_t run(Sim* s, int64_t n, int* done) {
   MultiPlan plan;
   // 2D: a node reaches the rows above and below, anywhere along them (periodic in x)
   multi_plan(n, s->D == 3 ? s->nz : 0, plane_blocks, 2.0 * per_row / Up::kThreads, bytes, blocks, (int)(s->step & 1),
-             &plan);
+             call.any_size, &plan);
   if (plan.steps < 2) return cudaSuccess;
+  if (!call.launch) {
+    *done = plan.steps;
+    return cudaSuccess;
+  }
   TpGrid p;
   p.g = tp::Grid{(int)s->nx, (int)s->ny, (int)s->nz, s->N};
   p.r = s->rates;
@@ -82,10 +86,10 @@ cudaError_t run(Sim* s, int64_t n, int* done) {
 
 }  // namespace
 
-cudaError_t tp_launch_steps(Sim* s, int64_t n, int* done) {
+cudaError_t tp_launch_steps(Sim* s, int64_t n, const StepsCall& call, int* done) {
   *done = 0;
   if (s->storage != LBM_F32 || !tp_pair_supported(s)) return cudaSuccess;
-  return s->D == 2 ? run<PairUp<2>>(s, n, done) : run<PairUp<3>>(s, n, done);
+  return s->D == 2 ? run<PairUp<2>>(s, n, call, done) : run<PairUp<3>>(s, n, call, done);
 }
 
 }  // namespace lbm

@@ -33,7 +33,7 @@ EXPORTS = (
     "lbm_init_fields", "lbm_step", "lbm_moments", "lbm_get_populations", "lbm_set_populations",
     "lbm_reduce", "lbm_step_totals", "lbm_step_totals_async", "lbm_mode_amplitude", "lbm_step_count", "lbm_status", "lbm_last_error",
     "lbm_reduce_noalloc", "lbm_mode_history", "lbm_alu_probe", "lbm_selftest_wait_timeout",
-    "lbm_set_active_planes", "lbm_sweep_kernel",
+    "lbm_set_active_planes", "lbm_sweep_kernel", "lbm_steps_per_launch",
 )
 
 
@@ -87,6 +87,8 @@ def load():
         L.lbm_set_active_planes.argtypes = [_vp, _i64, _i64]
         L.lbm_sweep_kernel.argtypes = [_vp]
         L.lbm_sweep_kernel.restype = ctypes.c_char_p
+        L.lbm_steps_per_launch.argtypes = [_vp, _i64]
+        L.lbm_steps_per_launch.restype = _i64
         L.lbm_alu_probe.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, _vp, _vp, _dp]
         L.lbm_last_error.argtypes = []
         L.lbm_last_error.restype = ctypes.c_char_p
@@ -209,6 +211,14 @@ def lbm_sweep_kernel(h):
     if name is None:
         raise LBMError(LBM_EINVAL, "NULL handle")
     return name.decode()
+
+
+def lbm_steps_per_launch(h, n):
+    """Steps that the first launch of lbm_step(h, n) takes (1: a launch per step)."""
+    steps = load().lbm_steps_per_launch(h, int(n))
+    if steps < 0:
+        _check(int(steps))
+    return steps
 
 
 def lbm_selftest_wait_timeout(h, polls):
@@ -395,6 +405,10 @@ class Simulation:
     def sweep_kernel(self):
         """Name of the sweep kernel that step() launches with the current settings."""
         return lbm_sweep_kernel(self.handle)
+
+    def steps_per_launch(self, n):
+        """Steps that the first launch of step(n) takes (1: a launch per step)."""
+        return lbm_steps_per_launch(self.handle, n)
 
     def set_active_planes(self, z_lo, z_count):
         """Sweep and reduce planes z_lo .. z_lo + z_count - 1 only (D3Q27 slabs)."""

@@ -56,6 +56,7 @@ def test_a_stream_with_few_sms_takes_the_same_steps(lbm, small_stream, lattice, 
     for stream in (None, small_stream):
         torch.cuda.synchronize()
         sim = lbm.Simulation(lattice, dims, [0.7, 1.0, 0.7, 1.0, 0.7][:3 if D == 2 else 5], storage="f32", stream=stream)
+        assert (sim.steps_per_launch(7) > 1) == (stream is None)
         sim.init_fields(rho, u)
         sim.step(7)
         assert sim.status() == lbm.LBM_OK and sim.step_count == 7
