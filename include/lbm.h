@@ -289,6 +289,16 @@ int64_t lbm_steps_per_launch(lbm_handle h, int64_t n);
  * status.  LBM_EINVAL for a NULL handle or polls out of range. */
 int lbm_selftest_wait_timeout(lbm_handle h, int polls);
 
+/* The same for the launch of several steps, whose tiles wait (with a poll limit)
+ * for neighbouring tiles of the step before: enqueues the launch that lbm_step(h, n)
+ * would begin with, on counters that no tile can bring up to what the second step
+ * waits for, and a limit of `polls` (1 .. 2^20).  The first step's tiles run, every
+ * wait runs out, the blocks return, the status word's timeout bit is set, and the
+ * populations are of no use any more: the next lbm_init_fields starts over.  The step
+ * count is left as it is.  LBM_EINVAL for a NULL handle, polls out of range, or a
+ * handle and n that lbm_steps_per_launch counts 1 for. */
+int lbm_selftest_steps_timeout(lbm_handle h, int64_t n, int polls);
+
 /* Arithmetic-throughput probe: the measured denominator of the ALU rooflines
  * of the sweeps that arithmetic, not memory, binds (the 37-velocity lattice in
  * FP32 / packed FP32x2, D2Q9 in FP64).  The paper has no counterpart; this is

@@ -782,6 +782,19 @@ int lbm_selftest_wait_timeout(lbm_handle h, int polls) {
   return cuda_check(cudaGetLastError(), "self-test wait kernel");
 }
 
+int lbm_selftest_steps_timeout(lbm_handle h, int64_t n, int polls) {
+  Sim* s = as_sim(h);
+  if (int rc = check_handle(s)) return rc;
+  if (polls < 1 || polls > (1 << 20)) return set_error(LBM_EINVAL, "polls must be in 1 .. 2^20");
+  StepsCall starved;
+  starved.polls = polls;
+  starved.starve = true;
+  int done = 0;
+  if (int rc = cuda_check(launch_steps(s, n, &done, starved), "self-test of several steps")) return rc;
+  if (done < 2) return set_error(LBM_EINVAL, "a call of %lld steps takes one step per launch here", (long long)n);
+  return LBM_OK;
+}
+
 int lbm_status(lbm_handle h) {
   Sim* s = as_sim(h);
   if (int rc = check_handle(s)) return rc;

@@ -63,6 +63,8 @@ struct HTables {
 struct StepsCall {
   bool any_size = false;  // also on grids that stay in L2 by themselves (tests)
   bool launch = true;     // else only count the steps
+  int polls = 1 << 20;    // limit of a tile's wait for its neighbours
+  bool starve = false;    // counters that no tile can bring up to what the next steps wait for (self-test)
 };
 
 struct Sim {

@@ -13,7 +13,9 @@
 // One counter per unit counts its finished tiles; a tile waits until those
 // counters reach s * tiles.  All waits point to earlier entries of the order and
 // all blocks are co-resident (cooperative launch), so the lowest unfinished tile
-// can always run; each wait is bounded all the same (bit 2 of the status word).
+// can always run; each wait is bounded all the same.  A wait that gives up sets bit 2
+// of the status word, and a word of this launch's own that ends the other waits (the
+// status word's bit may be left from an earlier launch, and this one be sound).
 //
 // Step s starts at position s * reach instead of 0 (units taken modulo the grid),
 // so that the periodic neighbours of its first unit have been finished by step
@@ -40,8 +42,8 @@ struct MultiPlan {
   int d_outer, d_mid, d_inner;  // the grid size as a step in (outer, mid, inner)
 };
 
-constexpr int kMultiCounters = kRedBlocks * 8 * (int)sizeof(double) / 4;  // they sit where reductions keep partials
-constexpr int kMultiWaitPolls = 1 << 20;
+// They sit where reductions keep partials, behind the word that says a wait has given up.
+constexpr int kMultiCounters = kRedBlocks * 8 * (int)sizeof(double) / 4 - 1;
 
 __device__ __forceinline__ int load_acquire(const int* p) {
   int v;
@@ -62,7 +64,8 @@ __device__ __forceinline__ void add_release(int* p, int v) {
 template <typename Up>
 __global__ void __launch_bounds__(Up::kThreads, Up::kMinBlocks)
     multi_step_kernel(const __grid_constant__ typename Up::Params prm, const __grid_constant__ MultiPlan plan,
-                      int* __restrict__ counters, int* __restrict__ status) {
+                      int* __restrict__ gave_up, int* __restrict__ status, int poll_limit) {
+  int* const counters = gave_up + 1;
   __shared__ int ready[2];
   const int tid = threadIdx.x, mids = plan.steps;
   // the block's first entry
@@ -110,12 +113,16 @@ __global__ void __launch_bounds__(Up::kThreads, Up::kMinBlocks)
       if (tid < 32) {
         int polls = 0;
         while (!satisfied(s, u)) {
-          if (++polls > kMultiWaitPolls || (polls % 1024 == 0 && (load_acquire(status) & 2))) {
+          // the whole warp or none of it: satisfied() takes all lanes
+          if (++polls > poll_limit || (polls % 1024 == 0 && __any_sync(0xffffffffu, load_acquire(gave_up) != 0))) {
             give_up = 1;
             break;
           }
         }
-        if (give_up && tid == 0) atomicOr(status, 2);
+        if (give_up && tid == 0) {
+          atomicOr(status, 2);
+          atomicExch(gave_up, 1);
+        }
       }
       if (__syncthreads_or(give_up)) return;
     }
@@ -228,17 +235,20 @@ inline void multi_plan(int64_t n, int64_t planes, int64_t plane_blocks, double r
 }
 
 template <typename Up>
-cudaError_t multi_launch(Sim* s, const typename Up::Params& prm, MultiPlan plan, int blocks) {
+cudaError_t multi_launch(Sim* s, const typename Up::Params& prm, MultiPlan plan, int blocks, const StepsCall& call) {
   const int64_t G = blocks;
   plan.d_inner = (int)(G % plan.tiles);
   plan.d_mid = (int)(G / plan.tiles % plan.steps);
   plan.d_outer = (int)(G / plan.tiles / plan.steps);
-  int* counters = reinterpret_cast<int*>(partials_buf(s));
-  cudaError_t e = cudaMemsetAsync(counters, 0, (size_t)plan.units * sizeof(int), s->stream);
+  int* gave_up = reinterpret_cast<int*>(partials_buf(s));
+  cudaError_t e = cudaMemsetAsync(gave_up, 0, (size_t)(1 + plan.units) * sizeof(int), s->stream);
+  if (e == cudaSuccess && call.starve)  // large negative numbers
+    e = cudaMemsetAsync(gave_up + 1, 0x80, (size_t)plan.units * sizeof(int), s->stream);
   if (e != cudaSuccess) return e;
   int* status = status_word(s);
+  int polls = call.polls;
   typename Up::Params p = prm;
-  void* args[] = {&p, &plan, &counters, &status};
+  void* args[] = {&p, &plan, &gave_up, &status, &polls};
   return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(multi_step_kernel<Up>), dim3((unsigned)G),
                                      dim3(Up::kThreads), args, 0, s->stream);
 }

@@ -75,7 +75,7 @@ cudaError_t run(Sim* s, int64_t n, const StepsCall& call, int* done) {
   p.f = s->pop;
   p.row = row_length(per_row);
   p.unit_blocks = plan.sub;
-  const cudaError_t e = multi_launch<Up>(s, p, plan, blocks);
+  const cudaError_t e = multi_launch<Up>(s, p, plan, blocks, call);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
     cudaGetLastError();  // not enough SMs for this stream: single sweeps need none
     return cudaSuccess;

@@ -33,7 +33,7 @@ EXPORTS = (
     "lbm_init_fields", "lbm_step", "lbm_moments", "lbm_get_populations", "lbm_set_populations",
     "lbm_reduce", "lbm_step_totals", "lbm_step_totals_async", "lbm_mode_amplitude", "lbm_step_count", "lbm_status", "lbm_last_error",
     "lbm_reduce_noalloc", "lbm_mode_history", "lbm_alu_probe", "lbm_selftest_wait_timeout",
-    "lbm_set_active_planes", "lbm_sweep_kernel", "lbm_steps_per_launch",
+    "lbm_set_active_planes", "lbm_sweep_kernel", "lbm_steps_per_launch", "lbm_selftest_steps_timeout",
 )
 
 
@@ -84,6 +84,7 @@ def load():
                                          _vp, _dp]
         L.lbm_mode_history.argtypes = [_vp, ctypes.c_int, _i64p, ctypes.c_int, _i64, _dp, _dp]
         L.lbm_selftest_wait_timeout.argtypes = [_vp, ctypes.c_int]
+        L.lbm_selftest_steps_timeout.argtypes = [_vp, _i64, ctypes.c_int]
         L.lbm_set_active_planes.argtypes = [_vp, _i64, _i64]
         L.lbm_sweep_kernel.argtypes = [_vp]
         L.lbm_sweep_kernel.restype = ctypes.c_char_p
@@ -224,6 +225,11 @@ def lbm_steps_per_launch(h, n):
 def lbm_selftest_wait_timeout(h, polls):
     """Enqueue the bounded-wait self-test (a wait that runs out on purpose)."""
     _check(load().lbm_selftest_wait_timeout(h, int(polls)))
+
+
+def lbm_selftest_steps_timeout(h, n, polls):
+    """Enqueue a launch of several steps whose waits run out on purpose."""
+    _check(load().lbm_selftest_steps_timeout(h, int(n), int(polls)))
 
 
 def lbm_alu_probe(kind, iters, blocks, threads, sink_ptr, stream_ptr=None):
