@@ -184,6 +184,12 @@ constexpr int kMultiMaxReach = 63;
 // Blocks of nodes per tile at most: more put the steps further apart (256^3: 504,
 // 476 and 525 us a step with 1, 2 and 4), fewer cost fences.
 constexpr int kMultiMaxSub = 2;
+// Steps per launch at most.  A launch holds every block slot of the GPU until its last
+// step, and L2 has room for many steps of a 2D grid or of small planes (4096 x 1801: 85
+// of 170 steps, 6.5 ms a launch; 256^3 has 3, 1.4 ms).  us a step in calls of 100 steps,
+// without a limit and so: D2Q9 2048^2 40.9 and 38.7, 4096^2 134.8 and 125.5, 4096 x 1801
+// 76.3 and 73.5, D3Q27 32 x 32 x 2000 58.4 and 54.5, 66 x 50 x 400 42.3 and 41.6.
+constexpr int kMultiMaxSteps = 32;
 
 // Plan of up to n steps over `planes` planes of `plane_blocks` blocks of nodes (3D),
 // or over one run of plane_blocks blocks (planes = 0, 2D) whose velocities reach
@@ -220,7 +226,7 @@ inline void multi_plan(int64_t n, int64_t planes, int64_t plane_blocks, double r
   };
   if (!fits(2)) return;
   int64_t T = 2;
-  while (T < n && fits(T + 1)) ++T;
+  while (T < n && T < kMultiMaxSteps && fits(T + 1)) ++T;
   const int64_t passes = (n + T - 1) / T;  // equal passes
   n = (n + passes - 1) / passes;
   if (n < 2 || n * tiles >= ((int64_t)1 << 30) || units * tiles >= ((int64_t)1 << 30)) return;

@@ -59,6 +59,7 @@ def test_which_grids_take_several_steps(lbm, monkeypatch, lattice, dims, storage
     assert sim.steps_per_launch(1) == 1
     if several:
         assert sim.steps_per_launch(2) == 2
+        assert sim.steps_per_launch(1000) <= 32
         monkeypatch.setenv("LBM_MULTI_STEP", "0")
         assert sim.steps_per_launch(20) == 1
     if several and lattice == "D3Q27":
