@@ -242,7 +242,7 @@ template <typename R>
 struct MomentModel {
   R no[5];      // minus the rates of orders 2..4
   R s;          // 1 / c^2
-  R basis;      // temperature tau of the Hermite basis the collision takes its moments in
+  R basis;      // temperature tau of the Hermite basis the collision takes its moments in (0: plain moments)
   R basis2x3;   // 3 tau^2
   R th_ref;     // theta_ref / c^2 - tau
   R th_iso;     // temperature of isothermal runs, 1 / c^2 - tau
@@ -252,14 +252,6 @@ struct MomentModel {
   int raw;      // relax in the absolute frame (the shifts to and from the relative frame are left out)
 };
 
-template <typename T>
-struct real_of {
-  using type = T;
-};
-template <>
-struct real_of<f2> {
-  using type = float;
-};
 template <typename T>
 __device__ __forceinline__ T spread(T x) {
   return x;
@@ -274,13 +266,6 @@ __device__ __forceinline__ bool in_range(float rho, float th, float usq, float l
 }
 __device__ __forceinline__ bool in_range(double rho, double th, double usq, double lim) {
   return rho > 0.0 && th > 0.0 && usq < lim;
-}
-__device__ __forceinline__ bool in_range(f2 rho, f2 th, f2 usq, float lim) {
-  float r0, r1, t0, t1, u0, u1;
-  unpack2(rho, r0, r1);
-  unpack2(th, t0, t1);
-  unpack2(usq, u0, u1);
-  return in_range(r0, t0, u0, lim) && in_range(r1, t1, u1, lim);
 }
 
 // theta rounded to 11 significant bits
@@ -297,9 +282,8 @@ inline double basis_temperature(double theta) {
 // errors it leaves in stress and heat flux (which recur every step on a slowly
 // varying state) are those of small numbers.
 template <typename T, int NC>
-__device__ __forceinline__ void to_basis(const T (&M)[NC], T (&H)[NC],
-                                         const MomentModel<typename real_of<T>::type>& m) {
-  const T t = spread<T>(m.basis), nt = neg_(t), nt3 = cst<T>(3.0) * nt, nt6 = nt3 + nt3;
+__device__ __forceinline__ void to_basis(const T (&M)[NC], T (&H)[NC], const MomentModel<T>& m) {
+  const T t = m.basis, nt = neg_(t), nt3 = cst<T>(3.0) * nt, nt6 = nt3 + nt3;
   H[0] = M[0];
   H[1] = M[1];
   H[2] = M[2];
@@ -312,7 +296,7 @@ __device__ __forceinline__ void to_basis(const T (&M)[NC], T (&H)[NC],
   H[cidx(0, 3)] = fma_(nt3, M[cidx(0, 1)], M[cidx(0, 3)]);
   if constexpr (NC == 15) {
     // x^4 - 6 tau x^2 + 3 tau^2 = x^4 - 6 tau (x^2 - tau) - 3 tau^2, and so on
-    const T q = spread<T>(m.basis2x3), t2 = t * t;
+    const T q = m.basis2x3, t2 = t * t;
     H[cidx(4, 0)] = fma_(neg_(q), M[0], fma_(nt6, H[cidx(2, 0)], M[cidx(4, 0)]));
     H[cidx(0, 4)] = fma_(neg_(q), M[0], fma_(nt6, H[cidx(0, 2)], M[cidx(0, 4)]));
     H[cidx(2, 2)] = fma_(neg_(t2), M[0], fma_(nt, H[cidx(2, 0)] + H[cidx(0, 2)], M[cidx(2, 2)]));
@@ -333,10 +317,9 @@ __device__ __forceinline__ void to_basis(const T (&M)[NC], T (&H)[NC],
 // in isothermal runs only), so order 2 is relaxed as half trace and half
 // difference: the collision then conserves the energy exactly too.
 template <typename T, int NC>
-__device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC],
-                                                  const MomentModel<typename real_of<T>::type>& m) {
+__device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC], const MomentModel<T>& m) {
   static_assert(NC == 10 || NC == 15, "truncation N = 3 or 4");
-  const T thr = spread<T>(m.th_ref);
+  const T thr = m.th_ref;
   const T drho = M[0];
   const T rho = cst<T>(1.0) + drho;
   const T irho = rcp_(rho);
@@ -351,7 +334,7 @@ __device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC]
   if (m.thermal) {
     de = half * fma_(tr, irho, neg_(usq));
   } else {
-    de = spread<T>(m.th_iso) - thr;
+    de = m.th_iso - thr;
     ht = half * fma_(neg_(jx), ux, fma_(neg_(jy), uy, tr)) - rho * de;
   }
   const T hd = half * fma_(neg_(jx), ux, fma_(jy, uy, M[cidx(2, 0)] - M[cidx(0, 2)]));
@@ -399,7 +382,7 @@ __device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC]
   }
   if (m.raw) ux = uy = cst<T>(0.0);
   const T u3x = cst<T>(3.0) * ux, u3y = cst<T>(3.0) * uy, u2x = ux + ux, u2y = uy + uy;
-  const T o2 = spread<T>(m.no[2]), o3 = spread<T>(m.no[3]);
+  const T o2 = m.no[2], o3 = m.no[3];
   const T a20 = A[cidx(2, 0)], a11 = A[cidx(1, 1)], a02 = A[cidx(0, 2)];
   // order 2: the shift leaves it
   const T k20 = o2 * a20, k11 = o2 * a11, k02 = o2 * a02;
@@ -417,7 +400,7 @@ __device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC]
   inc[cidx(0, 3)] = i03;
   if constexpr (NC == 15) {
     if (m.basis != 0) {  // order 4 as plain moments
-      const T t = spread<T>(m.basis), t3 = cst<T>(3.0) * t, t6 = t3 + t3;
+      const T t = m.basis, t3 = cst<T>(3.0) * t, t6 = t3 + t3;
       A[cidx(4, 0)] = fma_(t6, a20, A[cidx(4, 0)]);
       A[cidx(3, 1)] = fma_(t3, a11, A[cidx(3, 1)]);
       A[cidx(2, 2)] = fma_(t, a20 + a02, A[cidx(2, 2)]);
@@ -425,7 +408,7 @@ __device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC]
       A[cidx(0, 4)] = fma_(t6, a02, A[cidx(0, 4)]);
     }
     // order 4: K = A4 - [4] u A3 + [6] u u A2, back with [4] u K3 + [6] u u K2
-    const T o4 = spread<T>(m.no[4]);
+    const T o4 = m.no[4];
     const T u4x = u2x + u2x, u4y = u2y + u2y;
     const T x1 = ux * ux, y1 = uy * uy, xx = u3x * ux, yy = u3y * uy, xx6 = xx + xx, yy6 = yy + yy;
     const T xy3 = u3x * uy, xy4 = u4x * uy;
@@ -450,7 +433,7 @@ __device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC]
 #pragma unroll
     for (int q = 0; q < 5; ++q) k4[q] = fma_(o4, A[10 + q] - up[q], dn[q]);
     if (m.kext != 0) {  // K other than 6, or the absolute-frame relaxation of Hermite coefficients
-      const T e = spread<T>(m.kext) * spread<T>(m.s) * (o2 - o4);
+      const T e = m.kext * m.s * (o2 - o4);
       k4[0] = fma_(e, cst<T>(6.0) * a20, k4[0]);
       k4[1] = fma_(e, cst<T>(3.0) * a11, k4[1]);
       k4[2] = fma_(e, a20 + a02, k4[2]);
@@ -460,7 +443,7 @@ __device__ __forceinline__ bool moment_increments(const T (&M)[NC], T (&inc)[NC]
 #pragma unroll
     for (int q = 0; q < 5; ++q) inc[10 + q] = k4[q];
   }
-  return in_range(rho, th + spread<T>(m.basis), usq, m.usq_max);
+  return in_range(rho, th + m.basis, usq, m.usq_max);
 }
 
 // ---- correctly rounded transforms (FP32 storage) ----------------------------
@@ -493,15 +476,15 @@ __device__ __forceinline__ f2 cut(float x, float sigma) {
 }
 
 // The map's constants b = G^-1 M (the inverse Gram matrix of the monomials up to
-// order N under the rule's weights), as multiples of powers of c^2.
+// order 4 under the rule's weights), as multiples of powers of c^2.
 enum MapTerm {
   kT0, kT0_2, kT2_2, kT22, kT0_4, kT0_22, kT2_4, kT4_4, kT22_22, kT1, kT1_3, kT3_3, kT3_12, kT11, kT11_31, kT31_31,
   kMapTerms
 };
-__host__ __device__ constexpr double map_term(int t, int nc, double n) {  // n = c^2
-  return t == kT0 ? (nc == 15 ? 3.0 : 2.0)
-       : t == kT0_2 ? (nc == 15 ? -1.5 : -0.5) * n
-       : t == kT2_2 ? (nc == 15 ? 2.25 : 0.5) * n * n
+__host__ __device__ constexpr double map_term(int t, double n) {  // n = c^2
+  return t == kT0 ? 3.0
+       : t == kT0_2 ? -1.5 * n
+       : t == kT2_2 ? 2.25 * n * n
        : t == kT22 ? 0.25 * n * n
        : t == kT0_4 ? 0.125 * n * n
        : t == kT0_22 ? 0.25 * n * n
@@ -512,7 +495,7 @@ __host__ __device__ constexpr double map_term(int t, int nc, double n) {  // n =
        : t == kT1_3 ? -0.5 * n * n
        : t == kT3_3 ? n * n * n / 6.0
        : t == kT3_12 ? 0.5 * n * n * n
-       : t == kT11 ? (nc == 15 ? 4.0 : 1.0) * n * n
+       : t == kT11 ? 4.0 * n * n
        : t == kT11_31 ? -0.5 * n * n * n
                       : n * n * n * n / 6.0;
 }
@@ -520,9 +503,7 @@ struct Split {
   float h, l;
 };
 __host__ __device__ constexpr Split split_of(double x) { return Split{(float)x, (float)(x - (double)(float)x)}; }
-struct BuiltInSplitMap {
-  __device__ __forceinline__ Split at(int t) const { return split_of(map_term(t, kNC, kC * kC)); }
-};
+__device__ __forceinline__ Split map_split(int t) { return split_of(map_term(t, kC * kC)); }
 
 // s + c = sum of products of (x + xl) and h, s the rounded sum and c its error to second
 // order (the error terms are those of the rounded products)
@@ -547,13 +528,12 @@ struct Dot2 {
 
 // The polynomial's coefficients of the moments M + L (FP32 pairs) as unevaluated
 // sums s + c.  Pairs that only swap x and y share packed instructions.
-template <int NC, typename K>
-__device__ __forceinline__ void to_polynomial_exact(const float (&M)[NC], const float (&L)[NC], const K& k,
-                                                    float (&s)[NC], float (&c)[NC]) {
-  auto dot = [&](int i, int t) { return Dot2<float>(M[i], L[i], k.at(t)); };
-  auto add = [&](Dot2<float>& d, int i, int t) { d.add(M[i], L[i], k.at(t)); };
-  auto dot2 = [&](int i, int j, int t) { return Dot2<f2>(pack2(M[i], M[j]), pack2(L[i], L[j]), k.at(t)); };
-  auto add2 = [&](Dot2<f2>& d, int i, int j, int t) { d.add(pack2(M[i], M[j]), pack2(L[i], L[j]), k.at(t)); };
+__device__ __forceinline__ void to_polynomial_exact(const float (&M)[kNC], const float (&L)[kNC], float (&s)[kNC],
+                                                    float (&c)[kNC]) {
+  auto dot = [&](int i, int t) { return Dot2<float>(M[i], L[i], map_split(t)); };
+  auto add = [&](Dot2<float>& d, int i, int t) { d.add(M[i], L[i], map_split(t)); };
+  auto dot2 = [&](int i, int j, int t) { return Dot2<f2>(pack2(M[i], M[j]), pack2(L[i], L[j]), map_split(t)); };
+  auto add2 = [&](Dot2<f2>& d, int i, int j, int t) { d.add(pack2(M[i], M[j]), pack2(L[i], L[j]), map_split(t)); };
   auto put = [&](int i, const Dot2<float>& d) {
     s[i] = d.s;
     c[i] = d.c;
@@ -580,39 +560,36 @@ __device__ __forceinline__ void to_polynomial_exact(const float (&M)[NC], const 
   Dot2<f2> b12 = dot2(i12, i21, kT3_12);
   add2(b12, i10, i01, kT1_3);
   put2(i12, i21, b12);
-  if constexpr (NC == 15) {
-    constexpr int i40 = cidx(4, 0), i04 = cidx(0, 4), i22 = cidx(2, 2), i31 = cidx(3, 1), i13 = cidx(1, 3);
-    add(b00, i40, kT0_4);
-    add(b00, i04, kT0_4);
-    add(b00, i22, kT0_22);
-    add2(b2, i02, i20, kT22);
-    add2(b2, i40, i04, kT2_4);
-    add2(b2, i22, i22, kT2_4);
-    add(b11, i31, kT11_31);
-    add(b11, i13, kT11_31);
-    Dot2<f2> b4 = dot2(0, 0, kT0_4);
-    add2(b4, i20, i02, kT2_4);
-    add2(b4, i40, i04, kT4_4);
-    put2(i40, i04, b4);
-    Dot2<float> b22 = dot(0, kT0_22);
-    add(b22, i20, kT2_4);
-    add(b22, i02, kT2_4);
-    add(b22, i22, kT22_22);
-    put(i22, b22);
-    Dot2<f2> b31 = dot2(i31, i13, kT31_31);
-    add2(b31, i11, i11, kT11_31);
-    put2(i31, i13, b31);
-  }
+  constexpr int i40 = cidx(4, 0), i04 = cidx(0, 4), i22 = cidx(2, 2), i31 = cidx(3, 1), i13 = cidx(1, 3);
+  add(b00, i40, kT0_4);
+  add(b00, i04, kT0_4);
+  add(b00, i22, kT0_22);
+  add2(b2, i02, i20, kT22);
+  add2(b2, i40, i04, kT2_4);
+  add2(b2, i22, i22, kT2_4);
+  add(b11, i31, kT11_31);
+  add(b11, i13, kT11_31);
+  Dot2<f2> b4 = dot2(0, 0, kT0_4);
+  add2(b4, i20, i02, kT2_4);
+  add2(b4, i40, i04, kT4_4);
+  put2(i40, i04, b4);
+  Dot2<float> b22 = dot(0, kT0_22);
+  add(b22, i20, kT2_4);
+  add(b22, i02, kT2_4);
+  add(b22, i22, kT22_22);
+  put(i22, b22);
+  Dot2<f2> b31 = dot2(i31, i13, kT31_31);
+  add2(b31, i11, i11, kT11_31);
+  put2(i31, i13, b31);
   put(0, b00);
   put2(i20, i02, b2);
   put(i11, b11);
 }
 
 // hi + lo parts of the sums as M + L, M rounded
-template <int NC>
-__device__ __forceinline__ void round_parts(const f2 (&M2)[NC], float (&M)[NC], float (&L)[NC]) {
+__device__ __forceinline__ void round_parts(const f2 (&M2)[kNC], float (&M)[kNC], float (&L)[kNC]) {
 #pragma unroll
-  for (int k = 0; k < NC; ++k) {
+  for (int k = 0; k < kNC; ++k) {
     float hi, lo;
     unpack2(M2[k], hi, lo);
     M[k] = hi + lo;
@@ -623,14 +600,13 @@ __device__ __forceinline__ void round_parts(const f2 (&M2)[NC], float (&M)[NC], 
 constexpr int kMomentBits = 10;      // sum of e_x^4 over the rule: 660
 constexpr int kPolynomialBits = 8;   // sum of |e_x^p e_y^q| over p + q <= 4 at (3, 1): 179
 
-template <int NC>
-__device__ __forceinline__ void cut_polynomial(const float (&s)[NC], const float (&c)[NC], f2 (&b)[NC], int bits) {
+__device__ __forceinline__ void cut_polynomial(const float (&s)[kNC], const float (&c)[kNC], f2 (&b)[kNC]) {
   float mx = fabsf(s[0]);
 #pragma unroll
-  for (int k = 1; k < NC; ++k) mx = fmaxf(mx, fabsf(s[k]));
-  const float sigma = cut_at(mx, bits);
+  for (int k = 1; k < kNC; ++k) mx = fmaxf(mx, fabsf(s[k]));
+  const float sigma = cut_at(mx, kPolynomialBits);
 #pragma unroll
-  for (int k = 0; k < NC; ++k) {
+  for (int k = 0; k < kNC; ++k) {
     float hi, lo;
     unpack2(cut(s[k], sigma), hi, lo);
     b[k] = pack2(hi, lo + c[k]);
@@ -645,8 +621,7 @@ __device__ __forceinline__ float weigh(f2 p, Split w) {
 }
 
 // to_basis of the moments M + L, each H rounded once
-template <int NC>
-__device__ __forceinline__ void to_basis_exact(const float (&M)[NC], const float (&L)[NC], float (&H)[NC],
+__device__ __forceinline__ void to_basis_exact(const float (&M)[kNC], const float (&L)[kNC], float (&H)[kNC],
                                                const MomentModel<float>& m) {
   const float t = m.basis, t3 = 3.f * t, t6 = 6.f * t;
   auto sub = [&](float& h, float& l, float k, int i) {  // h + l -= k (M_i + L_i), k of at most 24 bits
@@ -669,27 +644,24 @@ __device__ __forceinline__ void to_basis_exact(const float (&M)[NC], const float
   less(cidx(1, 2), t, cidx(1, 0));
   less(cidx(2, 1), t, cidx(0, 1));
   less(cidx(0, 3), t3, cidx(0, 1));
-  if constexpr (NC == 15) {
-    less(cidx(3, 1), t3, cidx(1, 1));
-    less(cidx(1, 3), t3, cidx(1, 1));
-    auto fourth = [&](int c, float k1, int i1, float k2, int i2, float k0) {
-      float h = M[c], l = L[c];
-      sub(h, l, k1, i1);
-      if (i2 >= 0) sub(h, l, k2, i2);
-      sub(h, l, -k0, 0);
-      H[c] = h + l;
-    };
-    fourth(cidx(4, 0), t6, cidx(2, 0), 0.f, -1, m.basis2x3);
-    fourth(cidx(0, 4), t6, cidx(0, 2), 0.f, -1, m.basis2x3);
-    fourth(cidx(2, 2), t, cidx(2, 0), t, cidx(0, 2), t * t);
-  }
+  less(cidx(3, 1), t3, cidx(1, 1));
+  less(cidx(1, 3), t3, cidx(1, 1));
+  auto fourth = [&](int c, float k1, int i1, float k2, int i2, float k0) {
+    float h = M[c], l = L[c];
+    sub(h, l, k1, i1);
+    if (i2 >= 0) sub(h, l, k2, i2);
+    sub(h, l, -k0, 0);
+    H[c] = h + l;
+  };
+  fourth(cidx(4, 0), t6, cidx(2, 0), 0.f, -1, m.basis2x3);
+  fourth(cidx(0, 4), t6, cidx(0, 2), 0.f, -1, m.basis2x3);
+  fourth(cidx(2, 2), t, cidx(2, 0), t, cidx(0, 2), t * t);
 }
 
 // M + L <- M + L + inc for the orders that the collision changes
-template <int NC>
-__device__ __forceinline__ void add_increments(float (&M)[NC], float (&L)[NC], const float (&inc)[NC]) {
+__device__ __forceinline__ void add_increments(float (&M)[kNC], float (&L)[kNC], const float (&inc)[kNC]) {
 #pragma unroll
-  for (int k = 3; k < NC; ++k) {
+  for (int k = 3; k < kNC; ++k) {
     const float t = __fadd_rn(M[k], inc[k]);
     L[k] += two_sum_err(M[k], inc[k], t);
     M[k] = t;
@@ -709,15 +681,15 @@ __device__ __forceinline__ bool collide_exact(float (&v)[kQ], const MomentModel<
 #pragma unroll
     for (int i = 0; i < kQ; ++i) x[i] = cut(v[i], sigma);
     to_moments(x, M2);
-    round_parts<kNC>(M2, M, L);
+    round_parts(M2, M, L);
   }
   float H[kNC];
-  to_basis_exact<kNC>(M, L, H, m);
+  to_basis_exact(M, L, H, m);
   const bool ok = moment_increments<float, kNC>(H, inc, m);
-  add_increments<kNC>(M, L, inc);
-  to_polynomial_exact<kNC>(M, L, BuiltInSplitMap(), s, c);
+  add_increments(M, L, inc);
+  to_polynomial_exact(M, L, s, c);
   f2 b[kNC], x[kQ];
-  cut_polynomial<kNC>(s, c, b, kPolynomialBits);
+  cut_polynomial(s, c, b);
   from_polynomial<f2, true>(b, x);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) v[i] = weigh(x[i], split_of(w_of(i)));

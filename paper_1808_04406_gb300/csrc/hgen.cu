@@ -221,23 +221,23 @@ __global__ void __launch_bounds__(kHgThreads)
 // Shear wave on 80^2, rule E9-A, FP64: 48.2 -> 24.6 us a step (23.4 with
 // chained launches; 18 of them are the FP64 pipe: one warp on each of
 // 200 of the 608 SM partitions, 64 cycles per FP64 warp instruction).
-template <typename T, int NA, int NQ>
+template <int NA, int NQ>
 struct Orbits {
   int rest, xp[NA], xm[NA], yp[NA], ym[NA], pp[NQ], mp[NQ], pm[NQ], mm[NQ];  // velocity indices
   int da[NA], qa[NQ], qb[NQ];                                                // |e| of pairs, |e_x| and |e_y| of quadruples
-  T w0, pw[NA], qw[NQ];                                                      // weights
-  T p1[NA], p2[NA], p3[NA], p4[NA];                                          // powers of a
-  T a1[NQ], a2[NQ], a3[NQ], a4[NQ], b1[NQ], b2[NQ], b3[NQ], b4[NQ];          // a^p b^q of quadruples
-  T ab[NQ], a2b[NQ], ab2[NQ], a2b2[NQ], a3b[NQ], ab3[NQ];
-  T vp1[NA], vp2[NA], vp3[NA], vp4[NA];  // the same times the weight
-  T va1[NQ], va2[NQ], va3[NQ], va4[NQ], vb1[NQ], vb2[NQ], vb3[NQ], vb4[NQ];
-  T vab[NQ], va2b[NQ], vab2[NQ], va2b2[NQ], va3b[NQ], vab3[NQ];
+  double w0, pw[NA], qw[NQ];                                                 // weights
+  double p1[NA], p2[NA], p3[NA], p4[NA];                                     // powers of a
+  double a1[NQ], a2[NQ], a3[NQ], a4[NQ], b1[NQ], b2[NQ], b3[NQ], b4[NQ];     // a^p b^q of quadruples
+  double ab[NQ], a2b[NQ], ab2[NQ], a2b2[NQ], a3b[NQ], ab3[NQ];
+  double vp1[NA], vp2[NA], vp3[NA], vp4[NA];  // the same times the weight
+  double va1[NQ], va2[NQ], va3[NQ], va4[NQ], vb1[NQ], vb2[NQ], vb3[NQ], vb4[NQ];
+  double vab[NQ], va2b[NQ], vab2[NQ], va2b2[NQ], va3b[NQ], vab3[NQ];
 };
 
 // Fills o from the rule; false if the rule lacks a reflection, has other numbers of
 // orbits, or weights that differ within an orbit.
-template <typename T, int NA, int NQ>
-bool make_orbits(const HLattice& L, Orbits<T, NA, NQ>* o) {
+template <int NA, int NQ>
+bool make_orbits(const HLattice& L, Orbits<NA, NQ>* o) {
   int at[7][7];
   for (auto& r : at)
     for (int& k : r) k = -1;
@@ -247,7 +247,7 @@ bool make_orbits(const HLattice& L, Orbits<T, NA, NQ>* o) {
   int na = 0, nq = 0;
   o->rest = idx(0, 0);
   if (o->rest < 0) return false;
-  o->w0 = (T)L.w[o->rest];
+  o->w0 = L.w[o->rest];
   for (int a = 1; a <= 3; ++a) {
     const int xp = idx(a, 0), xm = idx(-a, 0), yp = idx(0, a), ym = idx(0, -a);
     if (xp < 0 && xm < 0 && yp < 0 && ym < 0) continue;
@@ -258,15 +258,15 @@ bool make_orbits(const HLattice& L, Orbits<T, NA, NQ>* o) {
     o->ym[na] = ym;
     o->da[na] = a;
     const double w = L.w[xp], d = a;
-    o->pw[na] = (T)w;
-    o->p1[na] = (T)d;
-    o->p2[na] = (T)(d * d);
-    o->p3[na] = (T)(d * d * d);
-    o->p4[na] = (T)(d * d * d * d);
-    o->vp1[na] = (T)(w * d);
-    o->vp2[na] = (T)(w * d * d);
-    o->vp3[na] = (T)(w * d * d * d);
-    o->vp4[na] = (T)(w * d * d * d * d);
+    o->pw[na] = w;
+    o->p1[na] = d;
+    o->p2[na] = d * d;
+    o->p3[na] = d * d * d;
+    o->p4[na] = d * d * d * d;
+    o->vp1[na] = w * d;
+    o->vp2[na] = w * d * d;
+    o->vp3[na] = w * d * d * d;
+    o->vp4[na] = w * d * d * d * d;
     ++na;
   }
   for (int b = 1; b <= 3; ++b)
@@ -282,46 +282,46 @@ bool make_orbits(const HLattice& L, Orbits<T, NA, NQ>* o) {
       o->qa[k] = a;
       o->qb[k] = b;
       const double w = L.w[pp], x = a, y = b;
-      o->qw[k] = (T)w;
-      o->a1[k] = (T)x;
-      o->a2[k] = (T)(x * x);
-      o->a3[k] = (T)(x * x * x);
-      o->a4[k] = (T)(x * x * x * x);
-      o->b1[k] = (T)y;
-      o->b2[k] = (T)(y * y);
-      o->b3[k] = (T)(y * y * y);
-      o->b4[k] = (T)(y * y * y * y);
-      o->ab[k] = (T)(x * y);
-      o->a2b[k] = (T)(x * x * y);
-      o->ab2[k] = (T)(x * y * y);
-      o->a2b2[k] = (T)(x * x * y * y);
-      o->a3b[k] = (T)(x * x * x * y);
-      o->ab3[k] = (T)(x * y * y * y);
-      o->va1[k] = (T)(w * x);
-      o->va2[k] = (T)(w * x * x);
-      o->va3[k] = (T)(w * x * x * x);
-      o->va4[k] = (T)(w * x * x * x * x);
-      o->vb1[k] = (T)(w * y);
-      o->vb2[k] = (T)(w * y * y);
-      o->vb3[k] = (T)(w * y * y * y);
-      o->vb4[k] = (T)(w * y * y * y * y);
-      o->vab[k] = (T)(w * x * y);
-      o->va2b[k] = (T)(w * x * x * y);
-      o->vab2[k] = (T)(w * x * y * y);
-      o->va2b2[k] = (T)(w * x * x * y * y);
-      o->va3b[k] = (T)(w * x * x * x * y);
-      o->vab3[k] = (T)(w * x * y * y * y);
+      o->qw[k] = w;
+      o->a1[k] = x;
+      o->a2[k] = x * x;
+      o->a3[k] = x * x * x;
+      o->a4[k] = x * x * x * x;
+      o->b1[k] = y;
+      o->b2[k] = y * y;
+      o->b3[k] = y * y * y;
+      o->b4[k] = y * y * y * y;
+      o->ab[k] = x * y;
+      o->a2b[k] = x * x * y;
+      o->ab2[k] = x * y * y;
+      o->a2b2[k] = x * x * y * y;
+      o->a3b[k] = x * x * x * y;
+      o->ab3[k] = x * y * y * y;
+      o->va1[k] = w * x;
+      o->va2[k] = w * x * x;
+      o->va3[k] = w * x * x * x;
+      o->va4[k] = w * x * x * x * x;
+      o->vb1[k] = w * y;
+      o->vb2[k] = w * y * y;
+      o->vb3[k] = w * y * y * y;
+      o->vb4[k] = w * y * y * y * y;
+      o->vab[k] = w * x * y;
+      o->va2b[k] = w * x * x * y;
+      o->vab2[k] = w * x * y * y;
+      o->va2b2[k] = w * x * x * y * y;
+      o->va3b[k] = w * x * x * x * y;
+      o->vab3[k] = w * x * y * y * y;
     }
   return na == NA && nq == NQ && 1 + 4 * NA + 4 * NQ == L.q;
 }
 
 // Node values by orbit, and calls of fn(value, velocity index, signed e_x, signed e_y, index of
 // the opposite velocity) for each.
-template <typename T, int NA, int NQ>
+template <int NA, int NQ>
 struct OrbitValues {
-  T r, xp[NA], xm[NA], yp[NA], ym[NA], pp[NQ], mp[NQ], pm[NQ], mm[NQ];
-  template <typename R, typename F>
-  __device__ __forceinline__ void each(const Orbits<R, NA, NQ>& o, F fn) {
+  double r, xp[NA], xm[NA], yp[NA], ym[NA], pp[NQ], mp[NQ], pm[NQ], mm[NQ];
+  template <typename F>
+  __device__ __forceinline__ void each(const Orbits<NA, NQ>& o, F fn) {
     fn(r, o.rest, 0, 0, o.rest);
 #pragma unroll
     for (int k = 0; k < NA; ++k) {
@@ -340,19 +340,17 @@ struct OrbitValues {
   }
 };
 
-template <typename T, typename R, int NA, int NQ, int NC>
-__device__ __forceinline__ void orbit_moments(const Orbits<R, NA, NQ>& o, const OrbitValues<T, NA, NQ>& v,
-                                              T (&M)[NC]) {
+template <int NA, int NQ, int NC>
+__device__ __forceinline__ void orbit_moments(const Orbits<NA, NQ>& o, const OrbitValues<NA, NQ>& v, double (&M)[NC]) {
   using h37::cidx;
-  using h37::spread;
 #pragma unroll
-  for (int c = 0; c < NC; ++c) M[c] = cst<T>(0.0);
+  for (int c = 0; c < NC; ++c) M[c] = 0.0;
   M[0] = v.r;
-  auto acc = [&](int c, R k, T x) { M[c] = fma_(spread<T>(k), x, M[c]); };
+  auto acc = [&](int c, double k, double x) { M[c] = fma_(k, x, M[c]); };
 #pragma unroll
   for (int k = 0; k < NQ; ++k) {
-    const T s1 = v.pp[k] + v.mm[k], d1 = v.pp[k] - v.mm[k], s2 = v.pm[k] + v.mp[k], d2 = v.pm[k] - v.mp[k];
-    const T ee = s1 + s2, oo = s1 - s2, oe = d1 + d2, eo = d1 - d2;
+    const double s1 = v.pp[k] + v.mm[k], d1 = v.pp[k] - v.mm[k], s2 = v.pm[k] + v.mp[k], d2 = v.pm[k] - v.mp[k];
+    const double ee = s1 + s2, oo = s1 - s2, oe = d1 + d2, eo = d1 - d2;
     M[0] = M[0] + ee;
     acc(cidx(2, 0), o.a2[k], ee);
     acc(cidx(0, 2), o.b2[k], ee);
@@ -373,7 +371,7 @@ __device__ __forceinline__ void orbit_moments(const Orbits<R, NA, NQ>& o, const 
   }
 #pragma unroll
   for (int k = 0; k < NA; ++k) {
-    const T sx = v.xp[k] + v.xm[k], dx = v.xp[k] - v.xm[k], sy = v.yp[k] + v.ym[k], dy = v.yp[k] - v.ym[k];
+    const double sx = v.xp[k] + v.xm[k], dx = v.xp[k] - v.xm[k], sy = v.yp[k] + v.ym[k], dy = v.yp[k] - v.ym[k];
     M[0] = M[0] + (sx + sy);
     acc(cidx(1, 0), o.p1[k], dx);
     acc(cidx(2, 0), o.p2[k], sx);
@@ -389,24 +387,23 @@ __device__ __forceinline__ void orbit_moments(const Orbits<R, NA, NQ>& o, const 
 }
 
 // w P(e) at every velocity
-template <typename T, typename R, int NA, int NQ, int NC>
-__device__ __forceinline__ void orbit_values(const Orbits<R, NA, NQ>& o, const T (&b)[NC], OrbitValues<T, NA, NQ>& v) {
+template <int NA, int NQ, int NC>
+__device__ __forceinline__ void orbit_values(const Orbits<NA, NQ>& o, const double (&b)[NC], OrbitValues<NA, NQ>& v) {
   using h37::cidx;
-  using h37::spread;
-  auto w0 = [&](R w, T x) { return spread<T>(w) * x; };
-  auto add = [&](R k, int c, T x) { return fma_(spread<T>(k), b[c], x); };
-  auto mul = [&](R k, int c) { return spread<T>(k) * b[c]; };
+  auto w0 = [&](double w, double x) { return w * x; };
+  auto add = [&](double k, int c, double x) { return fma_(k, b[c], x); };
+  auto mul = [&](double k, int c) { return k * b[c]; };
   v.r = w0(o.w0, b[0]);
 #pragma unroll
   for (int k = 0; k < NA; ++k) {
-    const T z = w0(o.pw[k], b[0]);
-    T ex = add(o.vp2[k], cidx(2, 0), z), ey = add(o.vp2[k], cidx(0, 2), z);
+    const double z = w0(o.pw[k], b[0]);
+    double ex = add(o.vp2[k], cidx(2, 0), z), ey = add(o.vp2[k], cidx(0, 2), z);
     if constexpr (NC == 15) {
       ex = add(o.vp4[k], cidx(4, 0), ex);
       ey = add(o.vp4[k], cidx(0, 4), ey);
     }
-    const T ox = add(o.vp3[k], cidx(3, 0), mul(o.vp1[k], cidx(1, 0)));
-    const T oy = add(o.vp3[k], cidx(0, 3), mul(o.vp1[k], cidx(0, 1)));
+    const double ox = add(o.vp3[k], cidx(3, 0), mul(o.vp1[k], cidx(1, 0)));
+    const double oy = add(o.vp3[k], cidx(0, 3), mul(o.vp1[k], cidx(0, 1)));
     v.xp[k] = ex + ox;
     v.xm[k] = ex - ox;
     v.yp[k] = ey + oy;
@@ -414,15 +411,15 @@ __device__ __forceinline__ void orbit_values(const Orbits<R, NA, NQ>& o, const T
   }
 #pragma unroll
   for (int k = 0; k < NQ; ++k) {
-    T ee = add(o.va2[k], cidx(2, 0), add(o.vb2[k], cidx(0, 2), w0(o.qw[k], b[0])));
-    T oo = mul(o.vab[k], cidx(1, 1));
+    double ee = add(o.va2[k], cidx(2, 0), add(o.vb2[k], cidx(0, 2), w0(o.qw[k], b[0])));
+    double oo = mul(o.vab[k], cidx(1, 1));
     if constexpr (NC == 15) {
       ee = add(o.va2b2[k], cidx(2, 2), add(o.va4[k], cidx(4, 0), add(o.vb4[k], cidx(0, 4), ee)));
       oo = add(o.va3b[k], cidx(3, 1), add(o.vab3[k], cidx(1, 3), oo));
     }
-    const T oe = add(o.va3[k], cidx(3, 0), add(o.vab2[k], cidx(1, 2), mul(o.va1[k], cidx(1, 0))));
-    const T eo = add(o.vb3[k], cidx(0, 3), add(o.va2b[k], cidx(2, 1), mul(o.vb1[k], cidx(0, 1))));
-    const T s1 = ee + oo, s2 = ee - oo, t1 = oe + eo, t2 = oe - eo;
+    const double oe = add(o.va3[k], cidx(3, 0), add(o.vab2[k], cidx(1, 2), mul(o.va1[k], cidx(1, 0))));
+    const double eo = add(o.vb3[k], cidx(0, 3), add(o.va2b[k], cidx(2, 1), mul(o.vb1[k], cidx(0, 1))));
+    const double s1 = ee + oo, s2 = ee - oo, t1 = oe + eo, t2 = oe - eo;
     v.pp[k] = s1 + t1;
     v.mm[k] = s1 - t1;
     v.pm[k] = s2 + t2;
@@ -447,39 +444,39 @@ struct HMap {
   __device__ __forceinline__ double n4s() const { return v[11]; }
   __device__ __forceinline__ double n4f() const { return v[12]; }
 };
-template <typename T, int NA, int NQ>
+template <int NA, int NQ>
 struct OrbitRule {
-  Orbits<T, NA, NQ> o;
+  Orbits<NA, NQ> o;
   HMap map;
 };
 
 template <int NA, int NQ, int NC>
-__device__ __forceinline__ bool orbit_update(const OrbitRule<double, NA, NQ>& rule, OrbitValues<double, NA, NQ>& v,
+__device__ __forceinline__ bool orbit_update(const OrbitRule<NA, NQ>& rule, OrbitValues<NA, NQ>& v,
                                              const h37::MomentModel<double>& m) {
   double M[NC], H[NC], inc[NC];
-  orbit_moments<double>(rule.o, v, M);
+  orbit_moments(rule.o, v, M);
   h37::to_basis<double, NC>(M, H, m);
   const bool ok = h37::moment_increments<double, NC>(H, inc, m);
 #pragma unroll
   for (int k = 3; k < NC; ++k) M[k] += inc[k];
   h37::to_polynomial<double, NC>(M, rule.map);
-  orbit_values<double>(rule.o, M, v);
+  orbit_values(rule.o, M, v);
   return ok;
 }
 
-template <bool ODD, typename T, int NA, int NQ>
-__device__ __forceinline__ void orbit_load(const T* __restrict__ f, const HGrid& g, const OrbitRule<T, NA, NQ>& rule,
-                                           int x, int y, OrbitValues<T, NA, NQ>& v) {
+template <bool ODD, int NA, int NQ>
+__device__ __forceinline__ void orbit_load(const double* __restrict__ f, const HGrid& g, const OrbitRule<NA, NQ>& rule,
+                                           int x, int y, OrbitValues<NA, NQ>& v) {
   const uint32_t node = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
-  v.each(rule.o, [&](T& val, int i, int ex, int ey, int opp) {
+  v.each(rule.o, [&](double& val, int i, int ex, int ey, int opp) {
     val = ODD ? f[(size_t)opp * g.N + hnbr(g, x, y, -ex, -ey)] : f[(size_t)i * g.N + node];
   });
 }
-template <bool ODD, typename T, int NA, int NQ>
-__device__ __forceinline__ void orbit_store(T* __restrict__ f, const HGrid& g, const OrbitRule<T, NA, NQ>& rule, int x,
-                                            int y, OrbitValues<T, NA, NQ>& v) {
+template <bool ODD, int NA, int NQ>
+__device__ __forceinline__ void orbit_store(double* __restrict__ f, const HGrid& g, const OrbitRule<NA, NQ>& rule, int x,
+                                            int y, OrbitValues<NA, NQ>& v) {
   const uint32_t node = (uint32_t)x + (uint32_t)g.nx * (uint32_t)y;
-  v.each(rule.o, [&](T& val, int i, int ex, int ey, int opp) {
+  v.each(rule.o, [&](double& val, int i, int ex, int ey, int opp) {
     if (ODD)
       f[(size_t)i * g.N + hnbr(g, x, y, ex, ey)] = val;
     else
@@ -488,15 +485,15 @@ __device__ __forceinline__ void orbit_store(T* __restrict__ f, const HGrid& g, c
 }
 
 // The sweep of hgen_sweep_kernel by orbits, threads walking the nodes in one dimension.
-template <typename T, int NC, int NA, int NQ, bool ODD>
+template <int NC, int NA, int NQ, bool ODD>
 __global__ void __launch_bounds__(kHgThreads)
-    hgen_orbit_kernel(T* __restrict__ f, HGrid g, const __grid_constant__ OrbitRule<T, NA, NQ> rule,
-                      const __grid_constant__ h37::MomentModel<T> m, int* __restrict__ status) {
+    hgen_orbit_kernel(double* __restrict__ f, HGrid g, const __grid_constant__ OrbitRule<NA, NQ> rule,
+                      const __grid_constant__ h37::MomentModel<double> m, int* __restrict__ status) {
   const uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
   chain_wait();
   if (node >= (uint32_t)g.N) return;
   const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
-  OrbitValues<T, NA, NQ> v;
+  OrbitValues<NA, NQ> v;
   orbit_load<ODD>(f, g, rule, x, y, v);
   if (!orbit_update<NA, NQ, NC>(rule, v, m)) atomicOr(status, 1);
   orbit_store<ODD>(f, g, rule, x, y, v);
@@ -530,7 +527,7 @@ struct HalfRule {
 };
 
 template <int NA, int NQ>
-void split_orbits(const OrbitRule<double, NA, NQ>& r, HalfRule<NA, (NQ + 1) / 2>* out) {
+void split_orbits(const OrbitRule<NA, NQ>& r, HalfRule<NA, (NQ + 1) / 2>* out) {
   const auto& o = r.o;
   *out = HalfRule<NA, (NQ + 1) / 2>{};
   out->map = r.map;
@@ -851,61 +848,57 @@ inline h37::Model hmodel(const Sim* s) {
   return m;
 }
 
-void fill_map(double c2, int, HMap* k) {
+void fill_map(double c2, HMap* k) {
   const double s = 1.0 / c2, n = c2;
   const double v[13] = {-s, -3.0 * s, -6.0 * s, s * s, 3.0 * s * s, n, n * n, 0.5 * n * n, 0.5 * n * n * n,
                         n * n * n / 6.0, 0.25 * n * n * n * n, n * n * n * n / 6.0, n * n * n * n / 24.0};
   for (int i = 0; i < 13; ++i) k->v[i] = v[i];
 }
 template <int NA, int NQ>
-bool fill_rule(const HLattice& L, int nc, OrbitRule<double, NA, NQ>* r) {
-  fill_map(L.c * L.c, nc, &r->map);
+bool fill_rule(const HLattice& L, OrbitRule<NA, NQ>* r) {
+  fill_map(L.c * L.c, &r->map);
   return make_orbits(L, &r->o);
 }
-template <typename T>
-h37::MomentModel<T> hmoment_model(const Sim* s) {
-  h37::MomentModel<T> m;
+h37::MomentModel<double> hmoment_model(const Sim* s) {
+  h37::MomentModel<double> m;
   const double sl = 1.0 / (s->hl.c * s->hl.c), tau = h37::basis_temperature(s->theta_ref * sl);
-  for (int n = 0; n < 5; ++n) m.no[n] = (T)-s->rates.w[n];
-  m.s = (T)sl;
-  m.basis = (T)tau;
-  m.basis2x3 = (T)(3.0 * tau * tau);
-  m.th_ref = (T)(s->theta_ref * sl - tau);
-  m.th_iso = (T)(sl - tau);
+  for (int n = 0; n < 5; ++n) m.no[n] = -s->rates.w[n];
+  m.s = sl;
+  m.basis = tau;
+  m.basis2x3 = 3.0 * tau * tau;
+  m.th_ref = s->theta_ref * sl - tau;
+  m.th_iso = sl - tau;
   m.kext = 0;
-  m.usq_max = (T)(4.0 * sl);
+  m.usq_max = 4.0 * sl;
   m.thermal = (s->flags & LBM_THERMAL) ? 1 : 0;
   m.raw = 0;
   return m;
 }
 
 // The orbit sweep if the rule has NA and NQ orbits of each kind; *taken says so.
-template <int S, int NC, int NA, int NQ>
+template <int NC, int NA, int NQ>
 cudaError_t orbit_sweep(Sim* s, int odd, bool* taken) {
-  using T = typename HStore<S>::type;
-  OrbitRule<T, NA, NQ> rule;
-  *taken = fill_rule(s->hl, NC, &rule);
+  OrbitRule<NA, NQ> rule;
+  *taken = fill_rule(s->hl, &rule);
   if (!*taken) return cudaSuccess;
+  double* f = static_cast<double*>(s->pop);
+  // two threads per node while that leaves at most one warp per SM partition: beyond, a
+  // partition would issue two shorter streams instead of one (us a step, one thread and
+  // two: 80^2 22.3 and 18.2, 64 x 152 22.3 and 18.1, 100^2 22.4 and 23.9, 139^2 25.4 and 33.1)
+  if (s->N <= (int64_t)4 * 152 * 16) {
+    constexpr int NH = (NQ + 1) / 2;
+    HalfRule<NA, NH> half;
+    split_orbits(rule, &half);
+    return launch_chained(odd ? hgen_half_kernel<NC, NA, NH, true> : hgen_half_kernel<NC, NA, NH, false>,
+                          dim3((unsigned)((2 * s->N + 31) / 32)), dim3(32), 0, s->stream, f, hgrid(s), half,
+                          hmoment_model(s), status_word(s));
+  }
   // the largest of 128, 64, 32 threads that gives every SM two blocks: small grids spread over all of them
   int t = kHgThreads;
   while (t > 32 && s->N < (int64_t)t * 2 * 152) t /= 2;
   const unsigned blocks = (unsigned)((s->N + t - 1) / t);
-  T* f = static_cast<T*>(s->pop);
-  if constexpr (S == LBM_F64) {
-    // two threads per node while that leaves at most one warp per SM partition: beyond, a
-    // partition would issue two shorter streams instead of one (us a step, one thread and
-    // two: 80^2 22.3 and 18.2, 64 x 152 22.3 and 18.1, 100^2 22.4 and 23.9, 139^2 25.4 and 33.1)
-    if (s->N <= (int64_t)4 * 152 * 16) {
-      HalfRule<NA, (NQ + 1) / 2> half;
-      split_orbits(rule, &half);
-      constexpr int NH = (NQ + 1) / 2;
-      return launch_chained(odd ? hgen_half_kernel<NC, NA, NH, true> : hgen_half_kernel<NC, NA, NH, false>,
-                            dim3((unsigned)((2 * s->N + 31) / 32)), dim3(32), 0, s->stream, f, hgrid(s), half,
-                            hmoment_model<T>(s), status_word(s));
-    }
-  }
-  return launch_chained(odd ? hgen_orbit_kernel<T, NC, NA, NQ, true> : hgen_orbit_kernel<T, NC, NA, NQ, false>,
-                        dim3(blocks), dim3(t), 0, s->stream, f, hgrid(s), rule, hmoment_model<T>(s), status_word(s));
+  return launch_chained(odd ? hgen_orbit_kernel<NC, NA, NQ, true> : hgen_orbit_kernel<NC, NA, NQ, false>, dim3(blocks),
+                        dim3(t), 0, s->stream, f, hgrid(s), rule, hmoment_model(s), status_word(s));
 }
 
 template <int S, int Q, int NC, bool EXACT>
@@ -931,12 +924,12 @@ cudaError_t sweep_t(Sim* s, int odd) {
     bool taken = false;
     cudaError_t e;
     if constexpr (Q == 37) {
-      e = orbit_sweep<S, NC, 3, 6>(s, odd, &taken);
+      e = orbit_sweep<NC, 3, 6>(s, odd, &taken);
       if (taken) return e;
     } else {
-      e = orbit_sweep<S, NC, 2, 2>(s, odd, &taken);
+      e = orbit_sweep<NC, 2, 2>(s, odd, &taken);
       if (taken) return e;
-      e = orbit_sweep<S, NC, 1, 3>(s, odd, &taken);
+      e = orbit_sweep<NC, 1, 3>(s, odd, &taken);
       if (taken) return e;
     }
   }

@@ -176,8 +176,11 @@ int multi_resident_blocks(cudaStream_t stream) {
 
 // How much of the 129 MB L2 the populations between the first and the last step may
 // take (D3Q27 FP32 256^3: 476 us a step with 64 MB, 486 with 90), and the size up to
-// which a whole grid stays in L2 by itself (160 x 96 x 76, 126 MB: 39 us a step in
-// chained launches, 42 here; D2Q9 2048^2, 151 MB: 45 and 40).
+// which a whole grid stays in L2 by itself.  us a step in chained launches and here,
+// D3Q27: 96^3 (96 MB) 26.8 and 28.1, 100^3 (108 MB) 32.3 and 38.5, 104^3 (121 MB) 37.9
+// and 36.7, 108^3 (136 MB) 43.3 and 41.7, 128^3 68.2 and 59.3, 160^3 131.8 and 114.6, 192^3
+// 222 and 197, 256^3 524 and 479, 320^3 1023 and 965; D2Q9: 1600^2 (92 MB) 22.1 and 25.5,
+// 1900^2 (130 MB) 39.7 and 36.1, 2048^2 45.4 and 38.7.
 constexpr int64_t kMultiBytes = (int64_t)64 << 20;
 constexpr int64_t kResidentBytes = (int64_t)128 << 20;
 constexpr int kMultiMaxReach = 63;
