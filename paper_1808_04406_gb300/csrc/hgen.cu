@@ -579,7 +579,9 @@ __global__ void __launch_bounds__(32)
   const HalfOrbits<NA, NH>& o = rule.half[h];
   chain_wait();
   const bool in = (id >> 1) < (uint32_t)g.N;
-  const uint32_t node = in ? id >> 1 : 0u;  // threads past the grid take part in the exchange
+  // threads past the grid take part in the exchange, with the last node's values: it is of
+  // their own warp, whose stores come after all of its loads
+  const uint32_t node = in ? id >> 1 : (uint32_t)g.N - 1u;
   const int y = (int)(node / (uint32_t)g.nx), x = (int)(node - (uint32_t)y * (uint32_t)g.nx);
   auto nbr = [&](int ex, int ey) { return h ? hnbr(g, x, y, ey, ex) : hnbr(g, x, y, ex, ey); };
   auto load = [&](int i, int ex, int ey, int opp) {
