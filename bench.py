@@ -790,11 +790,13 @@ def run_batch(args):
 
 
 THERMAL_N, THERMAL_THETA0, THERMAL_PR = 1024, 1.2, 0.71
-# FP32 arithmetic of one 37-velocity thermal lattice update through the Hermite tables:
-# 2 x 515 FFMA + 172 FADD + 36 FMUL, the one-node kernel's executed counts (ncu, both
-# parities); 16-bit offsets add 37 + 37 FMUL for the w_i scaling.  (FP64 storage, through
-# raw moments: 2 x 211 FFMA + 188 FADD + 75 FMUL.)
-H37_FLOPS_PER_LUP = {8: 685.0, 4: 1238.0, 2: 1238.0 + 74.0}  # by element size
+# FP32 arithmetic of one 37-velocity thermal lattice update through the Hermite tables
+# (16-bit storage, FP32 with plain transforms): 2 x 515 FFMA + 172 FADD + 36 FMUL, the
+# one-node kernel's executed counts (ncu, both parities); 16-bit offsets add 37 + 37 FMUL
+# for the w_i scaling.  FP64 storage and the correctly rounded FP32 transforms go through
+# raw moments: no ALU fraction is given for them.
+H37_FLOPS_PER_LUP = 1238.0
+H37_SCALE_FLOPS = 74.0
 # FP32 ALU peak from unit counts: 128 FP32 FMA lanes per SM x 2 flop x SMs x SM clock.
 FP32_LANES_PER_SM = 128
 
@@ -928,7 +930,9 @@ def run_thermal(args):
            "traffic": None, "peak_kind": peak_kind, "algorithmic_bytes_per_launch": bpl * n * n}
     clocks = clk.summary()
     sm_mhz = clocks.get("sm_max_mhz") or 2070.0
-    flops = H37_FLOPS_PER_LUP[esize]
+    exact = esize == 4 and not args.fast_transforms
+    tables = esize == 2 or (esize == 4 and not exact)
+    flops = H37_FLOPS_PER_LUP + (H37_SCALE_FLOPS if esize == 2 else 0.0)
     # the sweep issues packed FP32x2 FMAs: its peak is the packed probe's (measured in this run)
     alu_peak = measure_alu_peak("f32x2")
     alu_achieved = flops * n * n / launch / 1e12
@@ -939,10 +943,11 @@ def run_thermal(args):
            "algorithmic_flops_per_launch": flops * n * n}
     # 16-bit populations of 1024^2 stay in L2: the FP32 arithmetic binds; FP32 populations stream from HBM
     roof = dict(alu if esize == 2 else hbm)
-    exact = esize == 4 and not args.fast_transforms
     roof["kernel"] = ("h37_sweep_kernel (one node per thread, correctly rounded FP32 transforms)" if exact
-                      else "h37_pair_kernel (two nodes per thread, packed FP32x2)")
-    roof["hbm" if esize == 2 else "alu"] = hbm if esize == 2 else alu
+                      else "h37_pair_kernel (two nodes per thread, packed FP32x2)" if tables
+                      else "h37_sweep_kernel (one node per thread, FP64)")
+    if tables:
+        roof["hbm" if esize == 2 else "alu"] = hbm if esize == 2 else alu
     line = {"metric": METRIC, "value": n * n * K / (ms * 1e-3) / 1e6, "unit": UNIT, "n_gpus": 1, "steps": K,
             "warmup": args.warmup, "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": args.storage or "f16", "data": "synthetic",
