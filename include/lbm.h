@@ -164,7 +164,12 @@ int lbm_init_fields(lbm_handle h, const void* rho, const void* u, const void* th
 /* Advance n >= 0 time steps: each is the collide-then-stream update of
  * Sec. II.C (Eq. omega, final update) in one sweep.  Asynchronous on the
  * handle's stream; n = 0 does nothing, n < 0 is LBM_EINVAL.  A node that turns
- * unphysical sets the status word (lbm_status) instead of stopping the run. */
+ * unphysical sets the status word (lbm_status) instead of stopping the run.
+ * On FP32 grids larger than L2 up to 32 of the n steps share one cooperative launch
+ * (lbm_steps_per_launch; lbm_mode_history too), which waits for all of the GPU's
+ * block slots and holds them to its end, some milliseconds at most: work on other
+ * streams runs before or after it, not between its steps.  Where it should run
+ * between them, step one at a time, or set LBM_MULTI_STEP=0 in the environment. */
 int lbm_step(lbm_handle h, int64_t n);
 
 /* Density, velocity (lattice units) and, if theta is not NULL, temperature at

@@ -886,7 +886,8 @@ cudaError_t orbit_sweep(Sim* s, int odd, bool* taken) {
   double* f = static_cast<double*>(s->pop);
   // two threads per node while that leaves at most one warp per SM partition: beyond, a
   // partition would issue two shorter streams instead of one (us a step, one thread and
-  // two: 80^2 22.3 and 18.2, 64 x 152 22.3 and 18.1, 100^2 22.4 and 23.9, 139^2 25.4 and 33.1)
+  // two: 80^2 22.3 and 18.6, 64 x 152 22.3 and 18.1, 100^2 22.4 and 23.9, 139^2 25.4 and 33.1;
+  // 17 velocities on 80^2: E7-D 9.1 and 8.7, E7-A, whose 3 quadruples do not halve, 9.5 and 9.6)
   if (s->N <= (int64_t)4 * 152 * 16) {
     constexpr int NH = (NQ + 1) / 2;
     HalfRule<NA, NH> half;

@@ -1,6 +1,7 @@
 // Several steps per launch (multi_step.cuh) for the tensor-product lattices with
-// FP32 storage and even nx.  us a step in chained launches and here: D3Q27 256^3 524 and 480, D2Q9
-// 2048^2 45.4 and 39.6, 4096^2 176 and 131.  16-bit storage does not gain (D3Q27
+// FP32 storage and even nx.  us a step in chained launches and here, calls of 20 steps (3D)
+// and 100: D3Q27 128^3 68.2 and 59.3, 256^3 524 and 479, D2Q9 2048^2 45.4 and 38.7, 4096^2 176
+// and 125.  16-bit storage does not gain (D3Q27
 // 256^3 FP16: 356 with the plane-walking sweep, 451 here; D2Q9 4096^2 BF16 119 and
 // 152), nor does FP64, which its arithmetic binds (D2Q9 2048^2 854 and 958), nor odd
 // nx (241 x 200 x 200 322 with column pairs, 377 here), nor the 37-velocity lattices, whose code for both parities exceeds the instruction cache

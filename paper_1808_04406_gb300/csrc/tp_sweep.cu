@@ -55,7 +55,9 @@ __global__ void __launch_bounds__(kSweepThreads, LBM_SWEEP_MINB)
 // us a step with one node per thread and so: D3Q27 FP32 161 x 95 x 77 47.7 and 42.0,
 // 241 x 200 x 200 369 and 322, FP16 129 x 128 x 128 69.7 and 57.1; D2Q9 BF16 1023^2 9.9
 // and 9.3, but FP32 1023 x 1024 9.8 and 10.2.  Grids of less than a wave of blocks
-// keep their nodes on twice the threads (33^3 3.4 and 4.0).
+// keep their nodes on twice the threads (33^3 3.2 and 4.0, 161 x 95 x 4 3.9 and 4.2).  In the
+// second wave the two change over: FP32 53^3 (636 blocks) 6.4 and 7.6, 97 x 64 x 31 (775)
+// 7.5 and 8.4, 65^3 (1105) 10.4 and 10.3, 161 x 95 x 20 (1220) 11.0 and 10.8.
 template <int D, bool ODD>
 struct ColumnPair {
   uint32_t xo[3], zo[3];
